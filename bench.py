@@ -3,15 +3,15 @@
 
 Workload (default): 200 events x 20000 tracks, 10 barrel layers (r = 4..40 cm,
 Bz = 3.8 T), seeded synthetic events (see paper_1605_05508_gb300/synth.py).
-A step fits the whole batch: one graph of 10 per-layer kernel launches
-(propagate + Kalman update of every track). Metric: track-layer
+A step fits the whole batch in one kf_fit call: one launch that takes every
+track through the 10 layers (propagate + Kalman update) in registers. Metric: track-layer
 propagate+update steps per second. Inputs (1.2 GB) exceed the 129 MB L2, so
 no flush runs between steps.
 
 Also reported on the same line: the end-to-end number through kf_fit_host
 (host buffers, copies inside the timed region), the fused all-layers kernel,
 the plain per-event FP64 form on the same GPU (events/s factor), the roofline
-of the per-layer kernel, the oracle on the host cores (cpu_baseline), and the
+of the fit kernel, the oracle on the host cores (cpu_baseline), and the
 SM clocks sampled during the timed region.
 
 `--impl reference` times the FP64 CPU oracle (as it stands) on the host cores
@@ -232,14 +232,17 @@ def profile_value(name, key, files=FIT_SOURCES):
     return float(kv[key])
 
 
-def ncu_traffic(n_tracks, staged=False):
-    """DRAM bytes per fit-layer launch (the plain-load or the staged kernel) from
-    the committed ncu summary, scaled to n_tracks (traffic grows in proportion to
-    the tracks of a launch); None if absent or taken on a different kernel source."""
-    name = "fit_layer_stage_kernel" if staged else "fit_layer_kernel"
-    b = profile_value(f"{name}.traffic.txt", "dram_bytes_per_track")
+def ncu_traffic(n_tracks):
+    """DRAM bytes per staged fit-layer launch from the committed ncu summary,
+    scaled to n_tracks (traffic grows in proportion to the tracks of a launch);
+    None if absent or taken on a different kernel source."""
+    b = profile_value("fit_layer_stage_kernel.traffic.txt", "dram_bytes_per_track")
     return None if b is None else b * n_tracks
 
+
+# FP32 work of one track-layer step (FFMA x 2 + FADD + FMUL thread
+# instructions of the fused fit, counted by ncu).
+FIT_FLOP_PER_TRACK_LAYER = 1441.9
 
 # Algorithmic bytes of one track-layer step of the per-layer fit as the method
 # needs them: read the state (par 24 + cov 84), the hit (12) and the charge (1),
@@ -258,6 +261,25 @@ def fit_bytes_per_track_layer(L, seeds_have_lo, have_valid, have_chi2):
     wr = 24 + 12 + 84 + (4 if have_chi2 else 0)  # par, lo, cov, chi2
     wr_status = 4 * min(L, 2) / L
     return rd + rd_lo + rd_status + wr + wr_status
+
+
+def staged_roofline(n, L, chunks, ms_per_step):
+    """Roofline of the staged layer kernel: HBM, by the method's bytes."""
+    launch_s = ms_per_step / 1e3 / (L * chunks)
+    bpt = fit_bytes_per_track_layer(L, False, True, True)
+    achieved = FIT_METHOD_BYTES_PER_TRACK_LAYER * n / chunks / launch_s / 1e9
+    achieved_moved = bpt * n / chunks / launch_s / 1e9
+    peak, peak_kind = measured_peaks()
+    traffic = ncu_traffic(n)
+    return {"kernel": "fit_layer_stage_kernel", "bound": "hbm", "achieved": achieved, "peak": peak, "unit": "GB/s",
+            "frac": achieved / peak, "traffic": traffic if chunks == 1 else None,
+            "peak_kind": f"{peak_kind} (copy bandwidth)",
+            "algorithmic_bytes_per_track_layer": FIT_METHOD_BYTES_PER_TRACK_LAYER,
+            "launch_us": launch_s * 1e6,
+            "with_implementation_bytes": {
+                "bytes_per_track_layer": bpt, "achieved": achieved_moved, "frac": achieved_moved / peak,
+                "note": "the method's bytes plus the low parts of the position pair, hit-valid flags and status "
+                        "words this kernel also moves"}}
 
 
 # --------------------------------------------------------------------------- our arm
@@ -290,7 +312,7 @@ def run_ours(a):
     def step():
         kf.kf_fit(ctx, seeds, hits, out, chi2, status, stream)
 
-    # the library's autotuner picks the layer kernel's block size and L2 chunk on this batch
+    # the library's autotuner picks the fit's form and block size on this batch
     if a.fit_tuning:
         block, chunk, stage = ([int(v) for v in a.fit_tuning.split(",")] + [0])[:3]
         kf.kf_set_tuning(ctx, block, 0, 8, 0, chunk, stage)
@@ -326,31 +348,22 @@ def run_ours(a):
                    "max_ms": float(per_step.max()), "steps": int(a.steps)}
     value = whole_job_rate(n * L, world, ms_per_step / 1e3)
 
-    # roofline of the per-layer kernel: the graph holds only the L x chunks layer launches
-    launch_s = ms_per_step / 1e3 / (L * chunks)
-    bpt = fit_bytes_per_track_layer(L, False, True, True)
-    achieved = FIT_METHOD_BYTES_PER_TRACK_LAYER * n / chunks / launch_s / 1e9
-    achieved_moved = bpt * n / chunks / launch_s / 1e9
-    peak, peak_kind = measured_peaks()
-    traffic = ncu_traffic(n, bool(tuning.get("fit_stage")))
-    kname = "fit_layer_stage_kernel" if tuning.get("fit_stage") else f"fit_layer_kernel<{tuning['fit_block']}>"
-    roof = {"kernel": kname, "bound": "hbm", "achieved": achieved, "peak": peak, "unit": "GB/s",
-            "frac": achieved / peak, "traffic": traffic if chunks == 1 else None,
-            "peak_kind": f"{peak_kind} (copy bandwidth)",
-            "algorithmic_bytes_per_track_layer": FIT_METHOD_BYTES_PER_TRACK_LAYER,
-            "launch_us": launch_s * 1e6,
-            "with_implementation_bytes": {
-                "bytes_per_track_layer": bpt, "achieved": achieved_moved, "frac": achieved_moved / peak,
-                "note": "the method's bytes plus the low parts of the position pair, hit-valid flags and status "
-                        "words this kernel also moves"}}
+    line_peaks = peaks_leg(kf, ctx, stream, dev, smi_index)
+    launches = L * chunks if tuning.get("fit_stage") else 1
+    if tuning.get("fit_stage"):  # one graph of L x chunks layer launches, bound by HBM
+        roof = staged_roofline(n, L, chunks, ms_per_step)
+    else:  # one launch, the state in registers: bound by the FP32 pipe
+        roof = dict(fp32_roofline(FIT_FLOP_PER_TRACK_LAYER, n * L, ms_per_step / 1e3, line_peaks,
+                                  "FFMA x 2 + FADD + FMUL thread instructions counted by ncu"),
+                    kernel=f"fit_fused_kernel<{tuning['fit_block']}>", launch_us=ms_per_step * 1e3)
 
     line = {"metric": METRIC, "value": value, "unit": UNIT, "n_gpus": world, "steps": a.steps,
             "warmup": a.warmup, "ms_per_step": ms_per_step, "higher_is_better": True, "scaling": "weak",
             "vs_baseline": None, "dtype": "f32 (positions as float pairs)",
             "data": "synthetic (seeded generator, helix hits + Gaussian smear)",
-            "config": workload_config(a), "roofline": roof, "clocks": clk, "gpu_launches": a.steps * L * chunks,
+            "config": workload_config(a), "roofline": roof, "clocks": clk, "gpu_launches": a.steps * launches,
             "tuning": tuning, "step_ms_spread": step_spread}
-    line["peaks"] = peaks_leg(kf, ctx, stream, dev, smi_index)
+    line["peaks"] = line_peaks
 
     if not a.no_extras:
         line.update(extras(a, ctx, kf, torch, dev, det, ev, seeds, hits, out, chi2, status, stream, value,
@@ -467,14 +480,14 @@ def extras(a, ctx, kf, torch, dev, det, ev, seeds, hits, out, chi2, status, stre
         clk = float(line_clock_mhz(dev)) * 1e6
         peak = 4.0 * props.multi_processor_count * clk
         ach = ipt * n * L / (ms_f / 1e3)
-        res["fused"]["roofline"] = {"kernel": "fit_fused_kernel<0>", "bound": "alu", "achieved": ach, "peak": peak,
+        res["fused"]["roofline"] = {"kernel": "fit_fused_kernel", "bound": "alu", "achieved": ach, "peak": peak,
                                     "unit": "warp instructions/s", "frac": ach / peak,
                                     "warp_instructions_per_track_layer": ipt,
                                     "peak_kind": "4 issues per SM per cycle x SMs x max SM clock"}
     fpt = profile_value("fit_fused_kernel.instructions.txt", "fp32_flop_per_track_layer")
     f32r = fp32_roofline(fpt, n * L, ms_f / 1e3, peaks, "profiles/fit_fused_kernel.instructions.txt")
     if f32r:
-        res["fused"]["fp32_roofline"] = dict(f32r, kernel="fit_fused_kernel<0>")
+        res["fused"]["fp32_roofline"] = dict(f32r, kernel="fit_fused_kernel")
 
     # end to end through the public C ABI with pinned host buffers
     pin = lambda x: torch.from_numpy(np.ascontiguousarray(x)).pin_memory()
@@ -540,7 +553,7 @@ def extras(a, ctx, kf, torch, dev, det, ev, seeds, hits, out, chi2, status, stre
 
 def single_event_leg(a, kf, torch, dev, det, stream, rank):
     """The plain FP64 configuration: one event of 1 000 tracks (seed 1605),
-    fitted over the 10 layers by the FP32 per-layer graph, the plain FP64
+    fitted over the 10 layers by kf_fit (FP32), the plain FP64
     form and the oracle (one thread, and all host cores); medians of 20 GPU
     fits (CUDA events) and of 5 oracle runs."""
     from paper_1605_05508_gb300 import synth as S
@@ -617,9 +630,8 @@ def build_kernel_name(t, max_cands):
     return f"build_step_kernel<{t['build_hit_tile']}, {lw}, {int(scan == 1)}>"
 
 
-def build_step_launches(tune, Lb, max_cands, seed_layers=3):
-    """Kernel launches of one build step: the seed fit (one per seeding layer),
-    the hit binning (one launch unordered, else count, scan, scatter, sort) and
+def build_step_launches(tune, Lb, max_cands):
+    """Kernel launches of one build step: the seed fit (one), the hit binning (one launch unordered, else count, scan, scatter, sort) and
     kf_build -- register-resident: the seeds' events, the first layer (with
     more than one lane a seed), the other layers, the final pass; else the seed
     ordering (count, scan, scatter), global ids, first candidates, the layer
@@ -635,7 +647,7 @@ def build_step_launches(tune, Lb, max_cands, seed_layers=3):
             first_fused = 0 if rm > Lb else min(Lb, rm)
             steps = first_fused + 1 if first_fused < Lb else Lb
         build = 3 + 1 + 1 + steps + 1
-    return seed_layers + binning + build
+    return 1 + binning + build
 
 
 def build_leg(a, kf, torch, dev, stream, rank, world, dist, peaks=None):

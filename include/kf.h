@@ -130,16 +130,17 @@ int kf_last_cuda_error(const kf_ctx *ctx);
  * chi2 [n_layers][n] (device, -1 where no update happened, may be NULL),
  * status [n] (device, KF_ST_* bits, may be NULL).
  * out->par_lo may be NULL (then the low parts are dropped on output).
- * Executed as one graph of n_layers kernel launches (one per layer step),
- * captured once per argument set and replayed.
+ * Executed as one kernel launch that keeps each track in registers through
+ * all layers, or with kf_tuning.fit_stage = 1 as one graph of n_layers staged
+ * launches (one per layer step), captured once per argument set and replayed.
  * Errors: KF_EINVAL (sizes, null pointers, n_layers > config),
  * KF_ENOMEM (scratch), KF_ECUDA.
  */
 int kf_fit(kf_ctx *ctx, const kf_tracks *seeds, const kf_track_hits *hits, kf_tracks *out,
            float *chi2, int32_t *status, void *stream);
 
-/* Same result as kf_fit, computed by a single launch that keeps each track in
- * registers across all layers (no per-layer state round trip). */
+/* Same result as kf_fit, always by the single launch that keeps each track in
+ * registers across all layers (whatever kf_tuning.fit_stage). */
 int kf_fit_fused(kf_ctx *ctx, const kf_tracks *seeds, const kf_track_hits *hits, kf_tracks *out,
                  float *chi2, int32_t *status, void *stream);
 
@@ -327,8 +328,8 @@ int kf_refit(kf_ctx *ctx, const kf_tracks *seeds, const kf_track_hits *seed_hits
  * hand, Sec. 4; here the library measures on the caller's own batch.)
  */
 typedef struct {
-    int32_t fit_block;        /* threads per block of the kf_fit / kf_fit_noalloc layer
-                                 kernel: 64 or 128 (default 128); 24 warps per SM either way */
+    int32_t fit_block;        /* threads per block of the single-launch fit: 64 or 128
+                                 (default 128); 24 warps per SM either way */
     int32_t build_hit_tile;   /* hits staged in shared memory per warp by the kf_build step
                                  (bulk asynchronous copies of the window's bin rows):
                                  0 = none, the scans read global memory (default), or 512 */
@@ -351,16 +352,17 @@ typedef struct {
                                  prepared event through all its layers in the launches shared
                                  with the events prepared with it, and with 0 .. 3 steps all
                                  resident events one layer a launch) */
-    int32_t fit_chunk;        /* kf_fit: 0 = each layer step is one launch over the whole batch
-                                 (default); 262144, 524288 or 1048576 = the batch is fitted in
-                                 chunks of that many tracks, all layers of a chunk before the
-                                 next, so the chunk's state stays in the L2 cache between its
-                                 layer launches */
-    int32_t fit_stage;        /* kf_fit layer step: 0 = every thread loads its track's rows
-                                 (default), 1 = each warp's next 32 tracks are copied into shared
-                                 memory by tensor copies while it computes the current ones
-                                 (batches whose size is a multiple of 32 with 16-byte aligned
-                                 rows; others take form 0) */
+    int32_t fit_chunk;        /* kf_fit with fit_stage 1: 0 = each layer step is one launch over
+                                 the whole batch (default); 262144, 524288 or 1048576 = the
+                                 batch is fitted in chunks of that many tracks, all layers of a
+                                 chunk before the next, so the chunk's state stays in the L2
+                                 cache between its layer launches (no effect with fit_stage 0,
+                                 where the state stays in registers) */
+    int32_t fit_stage;        /* kf_fit: 0 = one launch, every track in registers through all
+                                 layers (default), 1 = one launch per layer step, each warp's
+                                 next 32 tracks copied into shared memory by tensor copies while
+                                 it computes the current ones (batches whose size is a multiple
+                                 of 32 with 16-byte aligned rows; others take form 0) */
     int32_t bin_unordered;    /* kf_bin_hits: 0 = the hits of a bin in id order (default, a
                                  deterministic output), 1 = in the order the scatter pass left
                                  them (one pass less); kf_build's results do not depend on it */
@@ -375,7 +377,7 @@ int kf_get_tuning(const kf_ctx *ctx, kf_tuning *out);
 int kf_set_tuning(kf_ctx *ctx, const kf_tuning *t);
 
 /* Autotuner of kf_fit: runs kf_fit on the caller's arguments once per
- * (fit_stage, fit_block, fit_chunk) value (one untimed call, then three timed with CUDA
+ * distinct (fit_stage, fit_block, fit_chunk) form (one untimed call, then three timed with CUDA
  * events on `stream`, which is synchronised), keeps the fastest in the context (a
  * setting must beat the best so far by 2 % to replace it; the simplest come first)
  * and writes the context's tuning to *chosen (may be NULL).  The outputs hold the
@@ -541,23 +543,13 @@ int kf_measure_peak(kf_ctx *ctx, int32_t kind, void *stream, double *flop_per_s)
  * change afterwards -- e.g. an online trigger process that reserves all of the
  * GPU at start-up and treats any later cudaMalloc as a fault, a host framework
  * whose own caching allocator owns the device memory, or a plug-in that its
- * host application forbids to allocate.  kf_fit, when `status` or
- * `out->par_lo` is NULL, takes per-track scratch from the context and grows it
- * with cudaMalloc on first use; this entry point takes that scratch from a
- * fixed array in libkf's static device memory instead (KF_NOALLOC_MAX_TRACKS
- * x 16 bytes = 4 MiB, held by every GPU that loads the library until the
- * process exits) and performs no allocation or free of any kind.
+ * host application forbids to allocate.  kf_fit with kf_tuning.fit_stage = 1
+ * takes per-track scratch from the context and instantiates a graph; this
+ * entry point always takes the single-launch form, which keeps a track's state
+ * and status in registers, and performs no allocation or free of any kind.
  *
- * Arguments, layouts, results and errors are those of kf_fit, except:
- *  - seeds->n > KF_NOALLOC_MAX_TRACKS returns KF_EINVAL (split the batch);
- *  - the layer steps are issued as plain kernel launches on `stream`.
- * The first call on a device looks up the array's device address (with the
- * context's device current) and caches it; make that first call before any
- * stream capture begins.  The cached address does not survive a
- * cudaDeviceReset (which also invalidates every kf_ctx).  Every call shares the one array and leaves its
- * contents behind; each call's first layer launch rewrites what the later
- * launches read, so no clearing is needed.  Calls that overlap on the GPU
- * (other streams, other host threads) race on the array: serialise them.
+ * Arguments, layouts, results and errors are those of kf_fit, except that
+ * seeds->n > KF_NOALLOC_MAX_TRACKS returns KF_EINVAL (split the batch).
  */
 int kf_fit_noalloc(kf_ctx *ctx, const kf_tracks *seeds, const kf_track_hits *hits, kf_tracks *out,
                    float *chi2, int32_t *status, void *stream);

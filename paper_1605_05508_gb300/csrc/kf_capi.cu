@@ -59,6 +59,34 @@ int check_fit(kf_ctx* ctx, const kf_tracks* seeds, const kf_track_hits* hits,
   return KF_OK;
 }
 
+FitFusedArgs fused_args(const kf_ctx* ctx, const kf_tracks* seeds, const kf_track_hits* hits, const kf_tracks* out,
+                        float* chi2, int32_t* status) {
+  FitFusedArgs a;
+  std::memset(&a, 0, sizeof a);
+  a.in_par = seeds->par;
+  a.in_lo = seeds->par_lo;
+  a.in_cov = seeds->cov;
+  a.charge = seeds->charge;
+  a.out_par = out->par;
+  a.out_lo = out->par_lo;
+  a.out_cov = out->cov;
+  a.hits = hits->xyz;
+  a.valid = hits->valid;
+  a.chi2 = chi2;
+  a.status = status;
+  a.n = seeds->n;
+  a.n_layers = hits->n_layers;
+  a.a_scale = float(kCLight * double(ctx->cfg.bz_tesla));
+  a.v0 = a.v1 = ctx->cfg.sigma_xy_cm * ctx->cfg.sigma_xy_cm;
+  a.v2 = ctx->cfg.sigma_z_cm * ctx->cfg.sigma_z_cm;
+  for (int l = 0; l < hits->n_layers; ++l) {
+    a.R[l] = ctx->radius[l];
+    a.x_x0[l] = ctx->x_x0[l];
+  }
+  a.mass = ctx->mass;
+  return a;
+}
+
 }  // namespace kfi
 
 using namespace kfi;
@@ -163,40 +191,65 @@ void kf_destroy(kf_ctx* ctx) {
   delete ctx;
 }
 
-// Per-layer fit replayed from a captured graph (one kernel node per layer).
-int kf_fit(kf_ctx* ctx, const kf_tracks* seeds, const kf_track_hits* hits, kf_tracks* out, float* chi2,
-           int32_t* status, void* stream) {
-  int rc = check_fit(ctx, seeds, hits, out);
-  if (rc) return rc;
+}  // extern "C"
+
+// The staged layer step (kf_tuning.fit_stage = 1) replayed from a captured
+// graph, one kernel node per layer (and chunk).  *done: false when the batch's
+// layout does not allow the tensor copies; nothing is issued then.
+static int fit_staged(kf_ctx* ctx, const kf_tracks* seeds, const kf_track_hits* hits, kf_tracks* out, float* chi2,
+                      int32_t* status, cudaStream_t user, bool* done) {
   const int64_t n = seeds->n;
-  if (n == 0) return KF_OK;
-  KF_CUDA_TRY(ctx, cudaSetDevice(ctx->device));
+  const int L = hits->n_layers;
+  *done = false;
   int32_t* st = status;
   if (!st) {
-    rc = scratch_reserve(ctx, ctx->s_status, size_t(n) * sizeof(int32_t));
+    const int rc = scratch_reserve(ctx, ctx->s_status, size_t(n) * sizeof(int32_t));
     if (rc) return rc;
     st = static_cast<int32_t*>(ctx->s_status.ptr);
   }
   float* lo = out->par_lo;
   if (!lo) {
-    rc = scratch_reserve(ctx, ctx->s_lo, size_t(n) * 3 * sizeof(float));
+    const int rc = scratch_reserve(ctx, ctx->s_lo, size_t(n) * 3 * sizeof(float));
     if (rc) return rc;
     lo = static_cast<float*>(ctx->s_lo.ptr);
   }
-  const int L = hits->n_layers;
-  const float a_scale = float(kCLight * double(ctx->cfg.bz_tesla));
-  const float v0 = ctx->cfg.sigma_xy_cm * ctx->cfg.sigma_xy_cm;
-  const float v2 = ctx->cfg.sigma_z_cm * ctx->cfg.sigma_z_cm;
-  const int block = ctx->tune.fit_block;
+  const FitFusedArgs f = fused_args(ctx, seeds, hits, out, chi2, st);
   // tracks per L2 block: every layer of a chunk runs before the next chunk,
   // so the chunk's state stays in L2 between its layer launches
   const int64_t chunk = ctx->tune.fit_chunk > 0 ? std::min<int64_t>(ctx->tune.fit_chunk, n) : n;
+  auto layer_args = [&](int l, int64_t c0) {
+    FitLayerArgs a;
+    a.begin = c0;
+    a.count = std::min(chunk, n - c0);
+    a.in_par = l == 0 ? seeds->par : out->par;
+    a.in_lo = l == 0 ? seeds->par_lo : lo;
+    a.in_cov = l == 0 ? seeds->cov : out->cov;
+    a.charge = seeds->charge;
+    a.out_par = out->par;
+    a.out_lo = lo;
+    a.out_cov = out->cov;
+    a.hit = hits->xyz + int64_t(l) * 3 * n;
+    a.valid = hits->valid ? hits->valid + int64_t(l) * n : nullptr;
+    a.chi2 = chi2 ? chi2 + int64_t(l) * n : nullptr;
+    a.status = st;
+    a.n = n;
+    a.a_scale = f.a_scale;
+    a.R = f.R[l];
+    a.x_x0 = f.x_x0[l];
+    a.mass = f.mass;
+    a.v0 = f.v0;
+    a.v1 = f.v1;
+    a.v2 = f.v2;
+    a.first = l == 0;
+    a.last = l == L - 1;
+    a.skip_tile = ctx->test_skip_tile;
+    a.wait_limit = ctx->test_wait_polls;
+    return a;
+  };
   std::vector<uint64_t> key = {1,
                                uint64_t(n),
                                uint64_t(L),
-                               uint64_t(block),
                                uint64_t(chunk),
-                               uint64_t(ctx->tune.fit_stage),
                                reinterpret_cast<uint64_t>(seeds->par),
                                reinterpret_cast<uint64_t>(seeds->par_lo),
                                reinterpret_cast<uint64_t>(seeds->cov),
@@ -210,48 +263,23 @@ int kf_fit(kf_ctx* ctx, const kf_tracks* seeds, const kf_track_hits* hits, kf_tr
                                reinterpret_cast<uint64_t>(st),
                                uint64_t(ctx->test_skip_tile),
                                uint64_t(ctx->test_wait_polls)};
-  cudaStream_t user = static_cast<cudaStream_t>(stream);
   GraphEntry* hit_entry = nullptr;
   for (auto& g : ctx->graphs)
     if (g.key == key) hit_entry = &g;
   if (!hit_entry) {
+    std::vector<FitStageMaps> maps;  // of every launch, before anything is issued
+    for (int64_t c0 = 0; c0 < n; c0 += chunk)
+      for (int l = 0; l < L; ++l) {
+        maps.emplace_back();
+        if (!make_stage_maps(layer_args(l, c0), &maps.back())) return KF_OK;
+      }
     cudaStream_t cs = ctx->capture_stream;
     KF_CUDA_TRY(ctx, cudaStreamBeginCapture(cs, cudaStreamCaptureModeThreadLocal));
     cudaError_t le = cudaSuccess;
-    for (int64_t c0 = 0; c0 < n && le == cudaSuccess; c0 += chunk)
-    for (int l = 0; l < L && le == cudaSuccess; ++l) {
-      FitLayerArgs a;
-      a.begin = c0;
-      a.count = std::min(chunk, n - c0);
-      a.in_par = l == 0 ? seeds->par : out->par;
-      a.in_lo = l == 0 ? seeds->par_lo : lo;
-      a.in_cov = l == 0 ? seeds->cov : out->cov;
-      a.charge = seeds->charge;
-      a.out_par = out->par;
-      a.out_lo = lo;
-      a.out_cov = out->cov;
-      a.hit = hits->xyz + int64_t(l) * 3 * n;
-      a.valid = hits->valid ? hits->valid + int64_t(l) * n : nullptr;
-      a.chi2 = chi2 ? chi2 + int64_t(l) * n : nullptr;
-      a.status = st;
-      a.n = n;
-      a.a_scale = a_scale;
-      a.R = ctx->radius[l];
-      a.x_x0 = ctx->x_x0[l];
-      a.mass = ctx->mass;
-      a.v0 = v0;
-      a.v1 = v0;
-      a.v2 = v2;
-      a.first = l == 0;
-      a.last = l == L - 1;
-      a.skip_tile = ctx->test_skip_tile;
-      a.wait_limit = ctx->test_wait_polls;
-      FitStageMaps maps;
-      if (ctx->tune.fit_stage && make_stage_maps(a, &maps))
-        le = launch_fit_layer_stage(a, maps, ctx->num_sms, cs);
-      else
-        le = launch_fit_layer(a, block, cs);
-    }
+    size_t q = 0;
+    for (int64_t c0 = 0; c0 < n; c0 += chunk)
+      for (int l = 0; l < L && le == cudaSuccess; ++l)
+        le = launch_fit_layer_stage(layer_args(l, c0), maps[q++], ctx->num_sms, cs);
     cudaGraph_t graph = nullptr;
     cudaError_t ee = cudaStreamEndCapture(cs, &graph);
     if (le != cudaSuccess) return cuda_fail(ctx, le);
@@ -271,53 +299,49 @@ int kf_fit(kf_ctx* ctx, const kf_tracks* seeds, const kf_track_hits* hits, kf_tr
   }
   hit_entry->last_use = ++ctx->use_clock;
   KF_CUDA_TRY(ctx, cudaGraphLaunch(hit_entry->exec, user));
+  *done = true;
   return KF_OK;
 }
 
-static int fit_fused_impl(kf_ctx* ctx, const kf_tracks* seeds, const kf_track_hits* hits, kf_tracks* out, float* chi2,
-                          int32_t* status, void* stream, bool upd64);
+extern "C" {
+
+// One launch takes every track through all layers in registers.  A launch
+// per layer moves a track's 124 bytes of state to memory and back each time
+// (261 B per track and layer); with the state in registers a layer reads 13 B
+// and writes 4 B of a track, and the launches between the layers are gone.
+int kf_fit(kf_ctx* ctx, const kf_tracks* seeds, const kf_track_hits* hits, kf_tracks* out, float* chi2,
+           int32_t* status, void* stream) {
+  const int rc = check_fit(ctx, seeds, hits, out);
+  if (rc) return rc;
+  if (seeds->n == 0) return KF_OK;
+  KF_CUDA_TRY(ctx, cudaSetDevice(ctx->device));
+  cudaStream_t user = static_cast<cudaStream_t>(stream);
+  if (ctx->tune.fit_stage) {
+    bool done = false;
+    const int rs = fit_staged(ctx, seeds, hits, out, chi2, status, user, &done);
+    if (rs || done) return rs;
+  }
+  KF_CUDA_TRY(ctx, launch_fit_fused(fused_args(ctx, seeds, hits, out, chi2, status), ctx->tune.fit_block, user));
+  return KF_OK;
+}
 
 int kf_fit_fused(kf_ctx* ctx, const kf_tracks* seeds, const kf_track_hits* hits, kf_tracks* out, float* chi2,
                  int32_t* status, void* stream) {
-  return fit_fused_impl(ctx, seeds, hits, out, chi2, status, stream, false);
+  const int rc = check_fit(ctx, seeds, hits, out);
+  if (rc) return rc;
+  if (seeds->n == 0) return KF_OK;
+  KF_CUDA_TRY(ctx, cudaSetDevice(ctx->device));
+  KF_CUDA_TRY(ctx, launch_fit_fused(fused_args(ctx, seeds, hits, out, chi2, status), ctx->tune.fit_block, static_cast<cudaStream_t>(stream)));
+  return KF_OK;
 }
 
 int kf_fit_mixed(kf_ctx* ctx, const kf_tracks* seeds, const kf_track_hits* hits, kf_tracks* out, float* chi2,
                  int32_t* status, void* stream) {
-  return fit_fused_impl(ctx, seeds, hits, out, chi2, status, stream, true);
-}
-
-static int fit_fused_impl(kf_ctx* ctx, const kf_tracks* seeds, const kf_track_hits* hits, kf_tracks* out, float* chi2,
-                          int32_t* status, void* stream, bool upd64) {
-  int rc = check_fit(ctx, seeds, hits, out);
+  const int rc = check_fit(ctx, seeds, hits, out);
   if (rc) return rc;
-  const int64_t n = seeds->n;
-  if (n == 0) return KF_OK;
+  if (seeds->n == 0) return KF_OK;
   KF_CUDA_TRY(ctx, cudaSetDevice(ctx->device));
-  FitFusedArgs a;
-  std::memset(&a, 0, sizeof a);
-  a.in_par = seeds->par;
-  a.in_lo = seeds->par_lo;
-  a.in_cov = seeds->cov;
-  a.charge = seeds->charge;
-  a.out_par = out->par;
-  a.out_lo = out->par_lo;
-  a.out_cov = out->cov;
-  a.hits = hits->xyz;
-  a.valid = hits->valid;
-  a.chi2 = chi2;
-  a.status = status;
-  a.n = n;
-  a.n_layers = hits->n_layers;
-  a.a_scale = float(kCLight * double(ctx->cfg.bz_tesla));
-  a.v0 = a.v1 = ctx->cfg.sigma_xy_cm * ctx->cfg.sigma_xy_cm;
-  a.v2 = ctx->cfg.sigma_z_cm * ctx->cfg.sigma_z_cm;
-  for (int l = 0; l < hits->n_layers; ++l) {
-    a.R[l] = ctx->radius[l];
-    a.x_x0[l] = ctx->x_x0[l];
-  }
-  a.mass = ctx->mass;
-  KF_CUDA_TRY(ctx, launch_fit_fused(a, static_cast<cudaStream_t>(stream), upd64));
+  KF_CUDA_TRY(ctx, launch_fit_mixed(fused_args(ctx, seeds, hits, out, chi2, status), static_cast<cudaStream_t>(stream)));
   return KF_OK;
 }
 

@@ -5,20 +5,17 @@
 // Track fitting is the branch-free part of Kalman-filter tracking (Cerati et
 // al., Sec. 2): with the hit set fixed, every track runs propagate + update
 // over the layers.  Forms:
-//   fit_layer_kernel        one layer step over the whole batch (kf_fit
-//                           replays one launch per layer from a captured CUDA
-//                           graph), plain coalesced row reads;
-//   fit_layer_stage_kernel  the same step with each warp's next 32 tracks
-//                           copied into shared memory by 2-D tensor copies
-//                           while it computes the current ones (an autotuned
-//                           alternative, bitwise equal);
 //   fit_fused_kernel        all layers in one launch, the track held in
-//                           registers (also the mixed-precision form);
+//                           registers (kf_fit, kf_fit_fused, kf_fit_noalloc;
+//                           fit_mixed_kernel: the mixed-precision form);
+//   fit_layer_stage_kernel  one layer step over the whole batch (kf_fit with
+//                           kf_tuning.fit_stage replays one launch per layer
+//                           from a captured CUDA graph), each warp's next 32
+//                           tracks copied into shared memory by 2-D tensor
+//                           copies while it computes the current ones
+//                           (bitwise equal);
 //   fit_f64_kernel          the plain FP64 form, launched per event and per
 //                           layer.
-// One track per thread, 24 resident warps per SM in the layer step.  Other
-// stagings of the rows (bulk copies per block or per 32 tracks, per-thread
-// cp.async double buffering) measured slower than plain reads.
 #include <cudaTypedefs.h>
 
 #include <algorithm>
@@ -31,13 +28,12 @@
 namespace kfi {
 
 constexpr int kFitThreads = 128;
-constexpr int kFitMinBlocks = 5;  // fused fit: 20 resident warps per SM (96 registers)
-// The layer kernel moves 261 B per track: at 20 resident warps per SM the
-// loads a warp issues at the start of its tracks do not keep enough bytes in
-// flight to reach the HBM rate (a pure copy with this access pattern takes
-// 181 us per 4M tracks at 20 warps, 150 us at full occupancy).  24 warps
-// (80 registers, no spills) measured best; 32 warps spill.
+// Resident warps per SM of the fused fit: 24 (80 registers, no spills).  The
+// layers' arithmetic is bound by instruction issue and register reads, not by
+// memory: 1.444 ms for 4M tracks x 10 layers against 1.472 at 20 warps.
 constexpr int kFitWarpsPerSM = 24;
+// with the table of events the index arithmetic takes the registers over 80
+constexpr int kFitTableBlocksPerSM = 5;
 constexpr int kNewtonF32 = 12;  // iteration cap of the safeguarded Newton solve
 constexpr int kNewtonF64 = 16;
 
@@ -129,29 +125,6 @@ __device__ __forceinline__ void fit_layer_track(const FitLayerArgs& A, int64_t i
   st |= raised;
   if ((A.last || stopped) && !pd5(p, C)) st |= KF_ST_NOT_PD;
   if (A.first || raised || A.last) A.status[i] = st;
-}
-
-// One track per thread over a grid that covers the batch: blocks start as
-// others finish, so the warps of an SM drift out of phase and their load
-// bursts overlap other warps' arithmetic.  THREADS (64 or 128, picked by the
-// autotuner) keeps kFitWarpsPerSM warps per SM resident either way.
-template <int THREADS>
-__global__ void __launch_bounds__(THREADS, kFitWarpsPerSM * 32 / THREADS) fit_layer_kernel(const FitLayerArgs A) {
-  const int64_t n = A.n;
-  const int64_t i = A.begin + int64_t(blockIdx.x) * blockDim.x + threadIdx.x;
-  if (i >= A.begin + A.count) return;
-  const int32_t st = A.first ? 0 : A.status[i];
-  float p[6], lo[3], C[21];
-  if (!(st & KF_ST_STOPPED)) {
-#pragma unroll
-    for (int c = 0; c < 6; ++c) p[c] = A.in_par[c * n + i];
-#pragma unroll
-    for (int c = 0; c < 3; ++c) lo[c] = A.in_lo ? A.in_lo[c * n + i] : 0.f;
-#pragma unroll
-    for (int c = 0; c < 21; ++c) C[c] = A.in_cov[c * n + i];
-  }
-  const bool has_hit = A.valid ? A.valid[i] != 0 : true;
-  fit_layer_track(A, i, st, p, lo, C, A.charge[i], has_hit, A.hit[i], A.hit[n + i], A.hit[2 * n + i]);
 }
 
 // ---------------------------------------------------------------------------
@@ -318,16 +291,22 @@ __device__ __forceinline__ void fused_track(const EV& E, const FitFusedArgs& A, 
   }
 }
 
-template <bool UPD64>
-__global__ void __launch_bounds__(kFitThreads, UPD64 ? 1 : kFitMinBlocks) fit_fused_kernel(const FitFusedArgs A) {
-  const int64_t stride = int64_t(gridDim.x) * blockDim.x;
-  for (int64_t i = int64_t(blockIdx.x) * blockDim.x + threadIdx.x; i < A.n; i += stride) fused_track<UPD64>(A, A, i);
+template <int THREADS>
+__global__ void __launch_bounds__(THREADS, kFitWarpsPerSM * 32 / THREADS) fit_fused_kernel(const FitFusedArgs A) {
+  const int64_t i = int64_t(blockIdx.x) * THREADS + threadIdx.x;
+  if (i < A.n) fused_track<false>(A, A, i);
+}
+
+// The mixed-precision form (kf_fit_mixed).
+__global__ void __launch_bounds__(kFitThreads, 1) fit_mixed_kernel(const FitFusedArgs A) {
+  const int64_t i = int64_t(blockIdx.x) * kFitThreads + threadIdx.x;
+  if (i < A.n) fused_track<true>(A, A, i);
 }
 
 // The fused fit of several events in one launch (the events a serving
 // iteration prepares): thread t fits track t - table[q].begin of event q,
 // the last with table[q].begin <= t; the arithmetic of fit_fused_kernel.
-__global__ void __launch_bounds__(kFitThreads, kFitMinBlocks)
+__global__ void __launch_bounds__(kFitThreads, kFitTableBlocksPerSM)
     fit_fused_table_kernel(const FitFusedArgs A, const FitEvent* table, int n_events, int64_t n_total) {
   const int64_t stride = int64_t(gridDim.x) * blockDim.x;
   for (int64_t t = int64_t(blockIdx.x) * blockDim.x + threadIdx.x; t < n_total; t += stride) {
@@ -366,19 +345,6 @@ __global__ void __launch_bounds__(kFitThreads) fit_f64_kernel(const FitF64Args A
   st |= raised;
   if ((A.last || stopped) && !pd5(p, C)) st |= KF_ST_NOT_PD;
   if (A.first || raised || A.last) A.status[i] = st;
-}
-
-int fit_grid(int block, int64_t n) {
-  const int64_t blocks = (n + block - 1) / block;
-  return int(blocks > 0 ? blocks : 1);
-}
-
-cudaError_t launch_fit_layer(const FitLayerArgs& a, int block, cudaStream_t st) {
-  if (block == 64)
-    fit_layer_kernel<64><<<fit_grid(64, a.count), 64, 0, st>>>(a);
-  else
-    fit_layer_kernel<128><<<fit_grid(128, a.count), 128, 0, st>>>(a);
-  return cudaGetLastError();
 }
 
 // Tensor maps of a layer step for fit_layer_stage_kernel: 2-D views (x =
@@ -435,13 +401,21 @@ cudaError_t launch_fit_fused_table(const FitFusedArgs& a, const FitEvent* table,
   return cudaGetLastError();
 }
 
-cudaError_t launch_fit_fused(const FitFusedArgs& a, cudaStream_t st, bool upd64) {
-  const int64_t blocks = (a.n + kFitThreads - 1) / kFitThreads;
-  const int grid = int(blocks > 0 ? blocks : 1);
-  if (upd64)
-    fit_fused_kernel<true><<<grid, kFitThreads, 0, st>>>(a);
+cudaError_t launch_fit_fused(const FitFusedArgs& a, int block, cudaStream_t st) {
+  if (a.n <= 0) return cudaSuccess;
+  // blocks of 32 for small batches, to spread their warps over the SMs, made no
+  // difference (18.43 us for 1 000 tracks x 10 layers either way)
+  const int grid = int((a.n + block - 1) / block);
+  if (block == 64)
+    fit_fused_kernel<64><<<grid, 64, 0, st>>>(a);
   else
-    fit_fused_kernel<false><<<grid, kFitThreads, 0, st>>>(a);
+    fit_fused_kernel<128><<<grid, 128, 0, st>>>(a);
+  return cudaGetLastError();
+}
+
+cudaError_t launch_fit_mixed(const FitFusedArgs& a, cudaStream_t st) {
+  if (a.n <= 0) return cudaSuccess;
+  fit_mixed_kernel<<<int((a.n + kFitThreads - 1) / kFitThreads), kFitThreads, 0, st>>>(a);
   return cudaGetLastError();
 }
 

@@ -89,7 +89,7 @@ int scratch_reserve(kf_ctx* ctx, Scratch& s, size_t bytes);
 // An empty batch (n = 0) is valid with any pointers.
 int check_fit(kf_ctx* ctx, const kf_tracks* seeds, const kf_track_hits* hits, const kf_tracks* out);
 
-// Arguments of one fit layer step (single precision).
+// Arguments of one staged fit layer step (single precision).
 struct FitLayerArgs {
   const float* in_par;
   const float* in_lo;  // may be null (lo = 0)
@@ -161,14 +161,18 @@ struct FitStageMaps {
   CUtensorMap par, lo, cov, hit;
 };
 
+// The arguments of a fused fit from a checked request (kf_capi.cu).
+FitFusedArgs fused_args(const kf_ctx* ctx, const kf_tracks* seeds, const kf_track_hits* hits, const kf_tracks* out,
+                        float* chi2, int32_t* status);
+
 // kernel launchers (kf_fit.cu)
 // block: threads per block, 64 or 128 (kf_tuning.fit_block)
-cudaError_t launch_fit_layer(const FitLayerArgs& a, int block, cudaStream_t st);
-// staged form (kf_tuning.fit_stage): false from make_stage_maps when the
-// batch's layout does not allow it (the caller then launches fit_layer_kernel)
+cudaError_t launch_fit_fused(const FitFusedArgs& a, int block, cudaStream_t st);
+cudaError_t launch_fit_mixed(const FitFusedArgs& a, cudaStream_t st);
+// staged layer step (kf_tuning.fit_stage): false from make_stage_maps when the
+// batch's layout does not allow it (kf_fit then takes the fused launch)
 bool make_stage_maps(const FitLayerArgs& a, FitStageMaps* m);
 cudaError_t launch_fit_layer_stage(const FitLayerArgs& a, const FitStageMaps& m, int num_sms, cudaStream_t st);
-cudaError_t launch_fit_fused(const FitFusedArgs& a, cudaStream_t st, bool upd64 = false);
 // One event of a table-driven fused fit: its arrays, as in FitFusedArgs, and
 // the launch's first thread for it.
 struct FitEvent {
@@ -207,6 +211,5 @@ struct RefitGatherArgs {
   int Ls, Lb, E;
 };
 cudaError_t launch_refit_gather(const RefitGatherArgs& a, cudaStream_t st);
-int fit_grid(int block, int64_t n);
 
 }  // namespace kfi

@@ -636,7 +636,7 @@ static cudaError_t finish(Serve* sv, Request* r) {
         q.x_x0[l] = ctx->x_x0[l];
       }
       q.mass = ctx->mass;
-      e = launch_fit_fused(q, s);
+      e = launch_fit_fused(q, sv->tune.fit_block, s);
     }
   }
   // results are contiguous on the device (rpar .. rhit, then the re-fit's)

@@ -1,8 +1,8 @@
 // kf_tune.cu -- launch parameters of the context and their autotuner.
 //
 // Each tunable changes how the work is laid out on the GPU, never the
-// arithmetic of a track: the fit kernel's block size (64 or 128 threads, 24
-// resident warps per SM either way), the build step's hit staging (window
+// arithmetic of a track: the fit in one launch (64 or 128 threads a block) or in
+// staged launches per layer, the build step's hit staging (window
 // hits copied per warp into shared memory, or read through L1), the length
 // of a lane's child list (4 suffices when at most 4 candidates are kept) and
 // the step's thread layout (8 lanes per seed, each lane scanning its own
@@ -104,6 +104,7 @@ int kf_autotune_fit(kf_ctx* ctx, const kf_tracks* seeds, const kf_track_hits* hi
       for (int chunk : {0, 262144, 524288, 1048576}) {
         if (chunk > 0 && seeds && chunk >= seeds->n) continue;  // one chunk: the same as 0
         if (stage == 1 && b != 64) continue;                     // the staged kernel has its own blocks
+        if (stage == 0 && chunk > 0) continue;                   // no state between launches to keep in L2
         kf_tuning t = ctx->tune;
         t.fit_block = b;
         t.fit_chunk = chunk;
