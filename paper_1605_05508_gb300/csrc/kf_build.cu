@@ -81,38 +81,72 @@ __device__ __forceinline__ int wrap_phi(int d) {  // to [-KF_BIN_PHI/2, KF_BIN_P
   return ((d + KF_BIN_PHI / 2) & (KF_BIN_PHI - 1)) - KF_BIN_PHI / 2;
 }
 
-// Window of a predicted candidate: S^-1 = (C_pos + V)^-1, and the eta rows
+// Approximate square root, reciprocal square root (a few ulp) and atan2 (within
+// 3e-6 rad) for the window bounds, which are widened by far more than that:
+// the correctly rounded forms and the library atan2f took several times the
+// instructions and a chain of dependent branches.
+__device__ __forceinline__ float sqrt_approx(float x) {
+  float r;
+  asm("sqrt.approx.ftz.f32 %0, %1;" : "=f"(r) : "f"(x));
+  return r;
+}
+__device__ __forceinline__ float rsqrt_approx(float x) {
+  float r;
+  asm("rsqrt.approx.ftz.f32 %0, %1;" : "=f"(r) : "f"(x));
+  return r;
+}
+// atan on [0, 1] by an odd polynomial of degree 11 (coefficients fitted for
+// the least maximal error, 1.7e-6), extended by the symmetries of atan2.
+// NaN for (0, 0) and non-finite arguments.
+__device__ __forceinline__ float atan2_approx(float y, float x) {
+  const float ax = fabsf(x), ay = fabsf(y);
+  const float t = __fdividef(fminf(ax, ay), fmaxf(ax, ay));
+  const float u = t * t;
+  float r = -0.011719135f;
+  r = fmaf(r, u, 0.05264735f);
+  r = fmaf(r, u, -0.11642648f);
+  r = fmaf(r, u, 0.19354038f);
+  r = fmaf(r, u, -0.33262283f);
+  r = fmaf(r, u, 0.9999772f);
+  r = r * t;
+  r = ay > ax ? 0.5f * kPi - r : r;
+  r = x < 0.f ? kPi - r : r;
+  return copysignf(r, y);
+}
+
+// Window of a predicted candidate: the eta rows
 // e0..e1 and phi bins fa0..fa1, fb0..fb1 (second part when the window wraps
 // around phi = +-pi) that can hold a hit with chi2 < cut at radius R; the
 // phi bins are those of a row of nphi bins over [-pi, pi) (KF_BIN_PHI, or
 // KF_BIN_PHI_FINE for the sub-bins), fa1 preset by the caller to nphi - 1.
 __device__ __forceinline__ void hit_window(const float p[6], const float lo[3], const float C[21], float R, float v0,
-                                           float v1, float v2, float cut, float Si[6], int& e0, int& e1, int& fa0,
-                                           int& fa1, int& fb0, int& fb1, int nphi = KF_BIN_PHI) {
-  kf::inverse_S(C, v0, v1, v2, Si);
+                                           float v1, float v2, float cut, int& e0, int& e1, int& fa0, int& fa1,
+                                           int& fb0, int& fb1, int nphi = KF_BIN_PHI) {
   const float X = p[0] + lo[0], Y = p[1] + lo[1], Z = p[2] + lo[2];
   // direction cosines of the position: they only scale the widths below,
   // which are widened by 0.1 %, so a reciprocal square root is exact enough
-  const float irr = rsqrtf(X * X + Y * Y);
+  const float irr = rsqrt_approx(X * X + Y * Y);
   const float cph = X * irr, sph = Y * irr;
   const float s00 = C[0] + v0, s10 = C[1], s11 = C[2] + v1, s22 = C[5] + v2;
   const float Stt = sph * sph * s00 - 2.f * sph * cph * s10 + cph * cph * s11;
   const float Snn = cph * cph * s00 + 2.f * sph * cph * s10 + sph * sph * s11;
-  const float wt = sqrtf(cut * fmaxf(Stt, 0.f));
-  const float wn = sqrtf(cut * fmaxf(Snn, 0.f));
-  const float wz = sqrtf(cut * fmaxf(s22, 0.f));
+  const float wt = sqrt_approx(cut * fmaxf(Stt, 0.f));
+  const float wn = sqrt_approx(cut * fmaxf(Snn, 0.f));
+  const float wz = sqrt_approx(cut * fmaxf(s22, 0.f));
   // A hit with chi2 < cut lies within wt of the prediction along the tangent,
   // wn along the normal and wz in z (chi2 >= (u.r)^2 / u^T S u for any unit
   // u), so its distance from the axis is between R - wn and
   // sqrt((R + wn)^2 + wt^2) and its phi within atan(wt / (R - wn)) of the
   // prediction's.  The bounds are widened by 0.1 % plus a small absolute
   // term -- far above the float rounding of the window, of the chi2 and of
-  // the hits' own bins -- and cover exactly the bins they reach; the phi
-  // half-width takes atan(x) <= x (x >= 0), a bound from above.
+  // the hits' own bins, and above the approximations' errors -- and cover
+  // exactly the bins they reach; the phi half-width takes atan(x) <= x
+  // (x >= 0), a bound from above.
   constexpr float kWiden = 1.001f;
   const float rin = R - wn * kWiden;
-  const float phic = atan2f(Y, X);
-  const float dphi = (rin > 0.5f * R && wt * kWiden < rin) ? (wt * kWiden / rin) * kWiden + 1e-6f : 10.f;
+  const float phic = atan2_approx(Y, X);
+  const float dphi =
+      (rin > 0.5f * R && wt * kWiden < rin) ? __fdividef(wt * kWiden, rin) * kWiden + 1.1e-5f : 10.f;
   if (dphi < 1.f && phic >= -kPi && phic <= kPi) {  // also false for NaN
     // the sub-bin scale is exactly twice the bin scale (a power of two), so a
     // hit's sub-bin halved is its bin
@@ -138,15 +172,15 @@ __device__ __forceinline__ void hit_window(const float p[6], const float lo[3], 
   e0 = 0;
   e1 = KF_BIN_ETA - 1;
   const float rlo = R - wn * kWiden - 1e-5f;
-  const float rhi = sqrtf((R + wn) * (R + wn) + wt * wt) * kWiden + 1e-5f;
+  const float rhi = sqrt_approx((R + wn) * (R + wn) + wt * wt) * kWiden + 1e-5f;
   if (rlo > 0.f) {
     const float zlo = Z - wz * kWiden - 1e-5f, zhi = Z + wz * kWiden + 1e-5f;
-    const float tmin = zlo >= 0.f ? zlo / rhi : zlo / rlo;
-    const float tmax = zhi >= 0.f ? zhi / rlo : zhi / rhi;
+    const float tmin = __fdividef(zlo, zlo >= 0.f ? rhi : rlo);
+    const float tmax = __fdividef(zhi, zhi >= 0.f ? rlo : rhi);
     // asinh by log(|t| + sqrt(t^2 + 1)) with the fast logarithm, widened by
     // 1e-5 in eta (far above that form's error): still a superset
-    e0 = eta_bin(copysignf(__logf(fabsf(tmin) + sqrtf(fmaf(tmin, tmin, 1.f))), tmin) - 1e-5f);
-    e1 = eta_bin(copysignf(__logf(fabsf(tmax) + sqrtf(fmaf(tmax, tmax, 1.f))), tmax) + 1e-5f);
+    e0 = eta_bin(copysignf(__logf(fabsf(tmin) + sqrt_approx(fmaf(tmin, tmin, 1.f))), tmin) - 1e-5f);
+    e1 = eta_bin(copysignf(__logf(fabsf(tmax) + sqrt_approx(fmaf(tmax, tmax, 1.f))), tmax) + 1e-5f);
   }
 }
 
@@ -273,7 +307,10 @@ __global__ void __launch_bounds__(kBuildThreads, kBuildBlocksPerSM) build_step_k
   const bool scan = active && !stopped;
   float Si[6];
   int e0 = 0, e1 = -1, fa0 = 0, fa1 = KF_BIN_PHI - 1, fb0 = 0, fb1 = -1;
-  if (scan) hit_window(p, lo, C, D.R, Args.v0, Args.v1, Args.v2, Args.cut, Si, e0, e1, fa0, fa1, fb0, fb1);
+  if (scan) {
+    kf::inverse_S(C, Args.v0, Args.v1, Args.v2, Si);
+    hit_window(p, lo, C, D.R, Args.v0, Args.v1, Args.v2, Args.cut, e0, e1, fa0, fa1, fb0, fb1);
+  }
   const int32_t* boff = D.bin_off + int64_t(seg) * (KF_NBINS + 1);
 
   // ---- warp union of the windows and staging (TILE > 0)
@@ -597,68 +634,121 @@ __device__ __forceinline__ bool scan_window(const float p[6], const float lo[3],
   return any;
 }
 
-// The same scan with a row's hits loaded kScanBatch at a time: all loads of a
-// batch are in flight before the first chi2 (the scan is bound by the round
-// trips of its dependent loads, not by its arithmetic).  Used by the
-// register-resident step: batches of 4 with one lane a seed, of 2 otherwise
-// (where the registers are needed elsewhere).
+// ---- register-resident step: a parent's children as (chi2 bits, hit position)
+//
+// All hit children of one parent have the same hit count and parent rank, so
+// among them the 64-bit key orders by (chi2_tot, hit id) alone: a lane's list
+// holds the bits of chi2_tot (compared unsigned, as in the key) and the hit's
+// position, half the registers of the keys, and the id -- in the hit's .w --
+// is looked at only when two chi2_tot are equal to the last bit.
+constexpr uint32_t kNoChild = 0xffffffffu;  // no float below the cut has these bits
+constexpr int kScanStage = 12;  // hits of a window staged in shared memory at a time (scan_children)
 
-template <int LW, int kScanBatch = 4>
-__device__ __forceinline__ bool scan_window_batched(const float p[6], const float lo[3], const float Si[6], int e0, int e1,
-                                            int fa0, int fa1, int fb0, int fb1, const int32_t* boff,
-                                            const float4* hs, float cut, int nh, float chi2tot, int k,
-                                            uint64_t (&L)[LW], int (&P)[LW], int nphi = KF_BIN_PHI) {
-  bool any = false;
-  const bool two = fb1 >= fb0;
-  int na0 = 0, na1 = 0, nb0 = 0, nb1 = 0;
-  if (e0 <= e1) {
-    const int32_t* q = boff + e0 * nphi;
-    na0 = q[fa0];
-    na1 = q[fa1 + 1];
-    if (two) {
-      nb0 = q[fb0];
-      nb1 = q[fb1 + 1];
+// Insert (x, u), the hit of id `id`, into the ascending list X/P (LW entries,
+// the last dropped).  Most parents have one compatible hit, so the first
+// insertion into an empty list is apart from the general one (measured with
+// the merge below: the window scan and the merge were half of the build's
+// instructions with 64-bit keys inserted the same way whatever the length).
+template <int LW>
+__device__ __forceinline__ void child_insert(uint32_t (&X)[LW], int (&P)[LW], uint32_t x, int u, int id,
+                                             const float4* hs) {
+  if (X[0] == kNoChild) {
+    X[0] = x;
+    P[0] = u;
+    return;
+  }
+  bool lt[LW];  // the new child goes before entry t
+  bool tie = false;
+#pragma unroll
+  for (int t = 0; t < LW; ++t) {
+    lt[t] = x < X[t];
+    tie |= x == X[t];
+  }
+  if (tie) {
+#pragma unroll
+    for (int t = 0; t < LW; ++t)
+      if (x == X[t]) lt[t] = id < __float_as_int(hs[P[t]].w);
+  }
+#pragma unroll
+  for (int t = LW - 1; t > 0; --t) {
+    if (lt[t - 1]) {
+      X[t] = X[t - 1];
+      P[t] = P[t - 1];
+    } else if (lt[t]) {
+      X[t] = x;
+      P[t] = u;
     }
   }
-  for (int er = e0; er <= e1; ++er) {
-    const int a0 = na0, na = na1 - na0, b0 = nb0, n = na + (nb1 - nb0);
-    if (er < e1) {
-      const int32_t* q = boff + (er + 1) * nphi;
-      na0 = q[fa0];
-      na1 = q[fa1 + 1];
-      if (two) {
-        nb0 = q[fb0];
-        nb1 = q[fb1 + 1];
+  if (lt[0]) {
+    X[0] = x;
+    P[0] = u;
+  }
+}
+
+// Chi2 scan of one predicted candidate's window (one thread): S^-1 =
+// (C_pos + V)^-1, then the pieces of rows e0..e1 -- bins fa0..fa1 of a row, then
+// fb0..fb1 where the window wraps around phi = +-pi; bin offsets `boff`, nphi
+// of them a row -- taken two at a time as one list of hits (most windows are
+// two rows and no wrap).  Every hit with chi2 < cut (and an id below the
+// segment limit) is inserted into the list (X, P) with chi2tot + chi2; the
+// list stays empty when there is none.
+// The scan is bound by the round trips of its dependent loads (offsets, then
+// hits), so all hits of a window, kScanStage at most, are in flight at once:
+// each thread copies its own into its column of `stage` (shared memory, slot
+// stride kResThreads) by cp.async, which holds no registers meanwhile; S^-1 is
+// computed while the offsets arrive, and the next pieces' offsets are fetched
+// beside the hits.
+__device__ __forceinline__ void cp_async16(float4* dst, const float4* src) {
+  asm volatile("cp.async.ca.shared.global [%0], [%1], 16;" ::"r"(smem_u32(dst)), "l"(src) : "memory");
+}
+template <int LW>
+__device__ __forceinline__ void scan_children(const float p[6], const float lo[3], const float C[21], float v0,
+                                              float v1, float v2, float Si[6], int e0, int e1, int fa0, int fa1,
+                                              int fb0, int fb1, const int32_t* boff, const float4* hs, float cut,
+                                              float chi2tot, uint32_t (&X)[LW], int (&P)[LW], int nphi,
+                                              float4* stage) {
+  const int two = fb1 >= fb0 ? 1 : 0;
+  const int np = (e1 - e0 + 1) << two;
+  int a0 = 0, b0 = 0, a1 = 0, b1 = 0;  // hits of the next two pieces
+  auto fetch = [&](int q, int& a, int& b) {
+    const int part = q & two;
+    const int32_t* row = boff + (e0 + (q >> two)) * nphi;
+    a = row[part ? fb0 : fa0];
+    b = row[(part ? fb1 : fa1) + 1];
+  };
+  if (np > 0) {
+    fetch(0, a0, b0);
+    fetch(min(1, np - 1), a1, b1);
+  }
+  kf::inverse_S(C, v0, v1, v2, Si);
+  for (int q = 0; q < np; q += 2) {
+    const int n0 = b0 - a0, n = n0 + (q + 1 < np ? b1 - a1 : 0);
+    const int s0 = a0, s1 = a1 - n0;
+    for (int w0 = 0; w0 < n; w0 += kScanStage) {
+      const int m = min(n - w0, kScanStage);
+#pragma unroll 1
+      for (int i = 0; i < m; ++i) {
+        const int v = w0 + i;
+        cp_async16(stage + i * kResThreads, hs + (v + (v < n0 ? s0 : s1)));
       }
-    }
-    // the row's hits in batches of kScanBatch loads in flight
-    for (int v0 = 0; v0 < n; v0 += kScanBatch) {
-      float4 mb[kScanBatch];
-      int ub[kScanBatch];
-#pragma unroll
-      for (int i = 0; i < kScanBatch; ++i) {
-        const int v = v0 + i;
-        ub[i] = v < na ? a0 + v : b0 + (v - na);
-        if (v < n) mb[i] = hs[ub[i]];
-      }
-#pragma unroll
-      for (int i = 0; i < kScanBatch; ++i) {
-        if (v0 + i < n) {
-          const float4 m = mb[i];
-          const float r0 = (m.x - p[0]) - lo[0], r1 = (m.y - p[1]) - lo[1], r2 = (m.z - p[2]) - lo[2];
-          const float c2 = kf::chi2_of(r0, r1, r2, Si);
-          if (c2 < cut) {
-            const int id = __float_as_int(m.w);
-            if (id < KF_MAX_HITS_PER_SEGMENT) {
-              list_insert(L, P, make_key(nh + 1, chi2tot + c2, k, id + 1), ub[i]);
-              any = true;
-            }
-          }
+      asm volatile("cp.async.wait_all;" ::: "memory");
+#pragma unroll 1
+      for (int i = 0; i < m; ++i) {
+        const float4 h = stage[i * kResThreads];
+        const float r0 = (h.x - p[0]) - lo[0], r1 = (h.y - p[1]) - lo[1], r2 = (h.z - p[2]) - lo[2];
+        const float c2 = kf::chi2_of(r0, r1, r2, Si);
+        if (c2 < cut) {
+          const int id = __float_as_int(h.w), v = w0 + i;
+          if (id < KF_MAX_HITS_PER_SEGMENT)
+            child_insert(X, P, __float_as_uint(chi2tot + c2), v + (v < n0 ? s0 : s1), id, hs);
         }
       }
     }
+    if (q + 2 < np) {
+      fetch(q + 2, a0, b0);
+      fetch(min(q + 3, np - 1), a1, b1);
+    }
   }
-  return any;
 }
 
 // ---- candidate-packed step (scan scheme 2)
@@ -808,7 +898,8 @@ __global__ void __launch_bounds__(NT, kBuildBlocksPerSM * kBuildThreads / NT) bu
       if (!stopped) {
         float Si[6];
         int e0 = 0, e1 = -1, fa0 = 0, fa1 = KF_BIN_PHI - 1, fb0 = 0, fb1 = -1;
-        hit_window(p, lo, C, D.R, Args.v0, Args.v1, Args.v2, Args.cut, Si, e0, e1, fa0, fa1, fb0, fb1);
+        kf::inverse_S(C, Args.v0, Args.v1, Args.v2, Si);
+        hit_window(p, lo, C, D.R, Args.v0, Args.v1, Args.v2, Args.cut, e0, e1, fa0, fa1, fb0, fb1);
         any = scan_window(p, lo, Si, e0, e1, fa0, fa1, fb0, fb1, D.bin_off + int64_t(s_seg[sd]) * (KF_NBINS + 1),
                           D.hits + s_h0[sd], Args.cut, nh, chi2tot, k, L, P);
       }
@@ -933,65 +1024,95 @@ __global__ void __launch_bounds__(NT, kBuildBlocksPerSM * kBuildThreads / NT) bu
 // are a total order and every candidate goes through the same functions as in
 // the other layouts, so the results are bitwise theirs.
 
-// Segmented merge: the W lanes of a seed (lanes gbase .. gbase + W - 1, mask
-// seg) hold sorted lists (L, P) of their own children; the best max_cands
-// keys of the union are found rank by rank by a minimum over the segment,
-// taken with full-warp shuffles that rotate within the segment (offsets 1, 2
-// and 4 reach every lane of a segment of up to 8): every lane executes the
-// same shuffle, so segments of different seeds proceed in one instruction
-// (warp intrinsics with a different member mask per segment are issued once
-// per segment).  Lane k of the segment receives the k-th best (key, hit
-// position); every lane the number of children kept.  Lanes outside any
-// seed's segment (seg == 0) rotate onto themselves.
-template <int W, int LW>
-__device__ __forceinline__ void merge_segment(uint64_t (&L)[LW], int (&P)[LW], int max_cands, int k, int gbase,
-                                              unsigned seg, uint64_t& my_key, int& my_pos, int& n_win) {
-  const int lane = threadIdx.x & 31;
-  const bool in_seg = seg != 0u;
-  const int r1 = in_seg ? gbase + (k + 1) % W : lane;
-  const int r2 = in_seg ? gbase + (k + 2) % W : lane;
-  const int r4 = in_seg ? gbase + (k + 4) % W : lane;
-  // the rank loop stays rolled: the step is large enough that the warps
-  // stall on instruction fetch, and an unrolled merge costs more there than
-  // its loop overhead (measured: 1.70 against 1.79 ms per build at N = 6)
-#pragma unroll 1
-  for (int r = 0; r < W; ++r) {
-    if (r < max_cands) {  // uniform over the launch
-      uint64_t m = L[0];
-      if constexpr (W > 1) {
-        uint64_t o = __shfl_sync(kFull, m, r1);
-        m = o < m ? o : m;
-        if constexpr (W > 2) {
-          o = __shfl_sync(kFull, m, r2);
-          m = o < m ? o : m;
-        }
-        if constexpr (W > 4) {
-          o = __shfl_sync(kFull, m, r4);
-          m = o < m ? o : m;
-        }
-      }
-      const bool mine = L[0] == m && m != kNoKey;
-      const unsigned bal = __ballot_sync(kFull, mine) & seg;
-      const int wl = bal ? __ffs(bal) - 1 : lane;
-      const int wpos = __shfl_sync(kFull, P[0], wl);
-      if (mine) {
+// The kept children of a seed, one per lane: lane k of the seed's W lanes
+// (lanes gbase .. gbase + W - 1, mask seg) receives the k-th best.
+struct Winner {
+  uint32_t x;  // chi2_tot bits
+  int pos;     // hit position, -1: no hit
+  int meta;    // parent rank | hit count << 8, -1: fewer children than this rank
+};
+
+// rank[t] += the children of the seed's other lanes that come before entry t
+// of this lane, over the first D entries of every list: by full-warp shuffles
+// that rotate within the seed's lanes (every lane executes the same shuffle,
+// so all seeds of the warp proceed together).
+template <int W, int D>
+__device__ __forceinline__ void count_before(const uint32_t (&X)[W], int nhk, int k, int gbase, unsigned seg,
+                                             int (&rank)[W]) {
+  auto rotate = [&](int r) {
+    int ko = k + r;
+    ko = ko >= W ? ko - W : ko;
+    const int src = seg ? gbase + ko : int(threadIdx.x & 31);
+    const int nho = __shfl_sync(kFull, nhk, src);
+    uint32_t xo[D];
 #pragma unroll
-        for (int t = 0; t < LW - 1; ++t) {
-          L[t] = L[t + 1];
-          P[t] = P[t + 1];
-        }
-        L[LW - 1] = kNoKey;
-        P[LW - 1] = -1;
-      }
-      if (m != kNoKey) {
-        if (k == r) {
-          my_key = m;
-          my_pos = wpos;
-        }
-        ++n_win;
-      }
+    for (int t = 0; t < D; ++t) xo[t] = __shfl_sync(kFull, X[t], src);
+    // the other lane's children below `lim` come first: all of them when they
+    // have more hits, none when they have fewer (an empty entry never)
+    const uint32_t after = ko < k ? 1u : 0u;
+#pragma unroll
+    for (int t = 0; t < D; ++t) {
+      const uint32_t lim = nho == nhk ? X[t] + after : nho > nhk ? kNoChild : 0u;
+#pragma unroll
+      for (int o = 0; o < D; ++o) rank[t] += xo[o] < lim ? 1 : 0;
     }
+  };
+  if constexpr (D <= 2) {
+#pragma unroll
+    for (int r = 1; r < W; ++r) rotate(r);
+  } else {  // seldom: kept small
+#pragma unroll 1
+    for (int r = 1; r < W; ++r) rotate(r);
   }
+}
+
+// Segmented merge: the W lanes of a seed hold sorted lists (X, P) of their own
+// children, all with nhk hits; the children are ranked by (hits desc, chi2
+// asc, parent rank asc), the order inside a lane being that of its list.  A
+// child's rank is its place in its own list plus the number of children of the
+// other lanes before it (count_before), the longest list of the warp (mostly
+// two entries) setting how many are compared; the ranks below max_cands then
+// go to their lanes through shared memory.  Picking the minimum rank by
+// rank took 42 shuffles a layer at W = 6 and shifted the lists at every rank.
+template <int W>
+__device__ __forceinline__ void merge_children(const uint32_t (&X)[W], const int (&P)[W], int nhk, int max_cands,
+                                               int k, int gbase, unsigned seg, int4* slots, Winner& win,
+                                               int& n_win) {
+  const int lane = threadIdx.x & 31;
+  if constexpr (W == 1) {
+    win.x = X[0];
+    win.pos = P[0];
+    win.meta = X[0] != kNoChild ? nhk << 8 : -1;
+    n_win = win.meta >= 0 ? 1 : 0;
+    return;
+  }
+  // entries of the warp's longest list (uniform)
+  const bool deep1 = __any_sync(kFull, X[1] != kNoChild);
+  const bool deep2 = W > 2 && __any_sync(kFull, X[W > 2 ? 2 : 0] != kNoChild);
+  const bool deep3 = W > 3 && __any_sync(kFull, X[W > 3 ? 3 : 0] != kNoChild);
+  int rank[W];
+#pragma unroll
+  for (int t = 0; t < W; ++t) rank[t] = t;
+  if (!deep1)
+    count_before<W, 1>(X, nhk, k, gbase, seg, rank);
+  else if (!deep2)
+    count_before<W, 2>(X, nhk, k, gbase, seg, rank);
+  else if (!deep3)
+    count_before<W, (W < 3 ? W : 3)>(X, nhk, k, gbase, seg, rank);
+  else
+    count_before<W, W>(X, nhk, k, gbase, seg, rank);
+  slots[lane] = make_int4(0, -1, -1, 0);
+  __syncwarp();
+#pragma unroll
+  for (int t = 0; t < W; ++t)
+    if (X[t] != kNoChild && rank[t] < max_cands)
+      slots[gbase + rank[t]] = make_int4(int(X[t]), P[t], k | nhk << 8, 0);
+  __syncwarp();
+  const int4 w = slots[lane];
+  win.x = uint32_t(w.x);
+  win.pos = w.y;
+  win.meta = w.z;
+  n_win = __popc(__ballot_sync(kFull, w.z >= 0) & seg);
 }
 
 template <typename T>
@@ -1026,6 +1147,9 @@ template <int W, bool TABLE, bool MAT>
 __global__ void __launch_bounds__(kResThreads, resident_blocks_per_sm(W))
     build_resident_kernel(const __grid_constant__ BuildResidentArgs A) {
   constexpr int G = 32 / W;  // seeds per group
+  __shared__ float4 s_stage[kScanStage * kResThreads];
+  __shared__ int4 s_slots[W > 1 ? kResThreads : 1];
+  int4* const slots = s_slots + (W > 1 ? int(threadIdx.x & ~31u) : 0);
   const int lane = threadIdx.x & 31;
   const int g = lane / W, k = lane - g * W;
   // the seed's lanes (none for lanes past G * W)
@@ -1047,7 +1171,10 @@ __global__ void __launch_bounds__(kResThreads, resident_blocks_per_sm(W))
       while (q + 1 < A.n_batches && A.table[q + 1].group_begin <= gi) ++q;
     const ResidentBatch& B = TABLE ? A.table[q] : A.one;
     const int64_t S8 = B.S * kGroup;
-    const int64_t j = (gi - (TABLE ? B.group_begin : 0)) * G + g;
+    // a batch's groups from the last to the first: the binning has just written
+    // the hits in order, so the last events' are the ones still in L2
+    // (measured: the N = 1 kernel of 12 uneven events 202 against 213 us)
+    const int64_t j = (TABLE ? gi - B.group_begin : n_groups - 1 - gi) * G + g;
     const bool seed_ok = g < G && j < B.S;
     int e = 0, nc = 0;
     int64_t si = 0;  // seed index
@@ -1096,7 +1223,7 @@ __global__ void __launch_bounds__(kResThreads, resident_blocks_per_sm(W))
       const int64_t h0 = seed_ok ? B.seg_off[sg] : 0;
       bool stopped = (st & KF_ST_STOPPED) != 0;
       if (active && !stopped) {
-        const int r = kf::propagate<float, kNewtonBuild, true>(p, lo, C, a, A.R[l]);
+        const int r = kf::propagate<float, kNewtonBuild, true, true>(p, lo, C, a, A.R[l]);
         if (r) {
           st |= r;
           stopped = true;
@@ -1105,11 +1232,11 @@ __global__ void __launch_bounds__(kResThreads, resident_blocks_per_sm(W))
         }
       }
       float Si[6] = {0.f, 0.f, 0.f, 0.f, 0.f, 0.f};
-      uint64_t L[W];
+      uint32_t X[W];
       int P[W];
 #pragma unroll
       for (int t = 0; t < W; ++t) {
-        L[t] = kNoKey;
+        X[t] = kNoChild;
         P[t] = -1;
       }
       const bool win = active && !stopped;
@@ -1118,46 +1245,46 @@ __global__ void __launch_bounds__(kResThreads, resident_blocks_per_sm(W))
       const int32_t* boff =
           B.fine_off ? B.fine_off + sg * (KF_NBINS_FINE + 1) : B.bin_off + sg * (KF_NBINS + 1);
       int e0 = 0, e1 = -1, fa0 = 0, fa1 = nphi - 1, fb0 = 0, fb1 = -1;
-      if (win) hit_window(p, lo, C, A.R[l], A.v0, A.v1, A.v2, A.cut, Si, e0, e1, fa0, fa1, fb0, fb1, nphi);
-      // a row's hits loaded in batches: 4 with one lane a seed, 2 with more
-      // (measured: 4 is slower at W = 6, where the registers are needed elsewhere)
-      bool any = false;
       if (win) {
-        if constexpr (W == 1)
-          any = scan_window_batched(p, lo, Si, e0, e1, fa0, fa1, fb0, fb1, boff, B.hits + h0, A.cut, nh, chi2tot, k,
-                                    L, P, nphi);
-        else
-          any = scan_window_batched<W, 2>(p, lo, Si, e0, e1, fa0, fa1, fb0, fb1, boff, B.hits + h0, A.cut, nh,
-                                          chi2tot, k, L, P, nphi);
+        hit_window(p, lo, C, A.R[l], A.v0, A.v1, A.v2, A.cut, e0, e1, fa0, fa1, fb0, fb1, nphi);
+        scan_children(p, lo, C, A.v0, A.v1, A.v2, Si, e0, e1, fa0, fa1, fb0, fb1, boff, B.hits + h0, A.cut, chi2tot, X,
+                      P, nphi, s_stage + threadIdx.x);
       }
       // no compatible hit (or a stopped candidate): one child without a hit
-      if (active && !any) list_insert(L, P, make_key(nh, chi2tot, k, 0), -1);
+      int nhk = nh + 1;
+      if (active && X[0] == kNoChild) {
+        X[0] = __float_as_uint(chi2tot);
+        nhk = nh;
+      }
       // clone engine: the seed's best max_cands children
-      uint64_t my_key = kNoKey;
-      int my_pos = -1;
-      n_win = 0;
-      merge_segment<W, W>(L, P, A.max_cands, k, g * W, seg, my_key, my_pos, n_win);
+      Winner w;
+      merge_children<W>(X, P, nhk, A.max_cands, k, g * W, seg, slots, w, n_win);
       // materialise: lane k takes its winner's parent prediction and S^-1
-      const int src = k < n_win ? g * W + int((my_key >> 21) & 7u) : lane;
+      const int src = w.meta >= 0 ? g * W + (w.meta & 7) : lane;
       float q[6], ql[3], qC[21], qS[6];
+      auto take = [&](auto v) {
+        if constexpr (W > 1)
+          return __shfl_sync(kFull, v, src);
+        else
+          return v;  // one lane a seed: its own prediction
+      };
 #pragma unroll
-      for (int c = 0; c < 6; ++c) q[c] = __shfl_sync(kFull, p[c], src);
+      for (int c = 0; c < 6; ++c) q[c] = take(p[c]);
 #pragma unroll
-      for (int c = 0; c < 3; ++c) ql[c] = __shfl_sync(kFull, lo[c], src);
+      for (int c = 0; c < 3; ++c) ql[c] = take(lo[c]);
 #pragma unroll
-      for (int c = 0; c < 21; ++c) qC[c] = __shfl_sync(kFull, C[c], src);
+      for (int c = 0; c < 21; ++c) qC[c] = take(C[c]);
 #pragma unroll
-      for (int c = 0; c < 6; ++c) qS[c] = __shfl_sync(kFull, Si[c], src);
-      const int32_t pst = __shfl_sync(kFull, st, src);
-      const int pstopped = __shfl_sync(kFull, int(stopped), src);
-      active = seed_ok && k < n_win;
+      for (int c = 0; c < 6; ++c) qS[c] = take(Si[c]);
+      const int32_t pst = take(st);
+      const int pstopped = take(int(stopped));
+      active = seed_ok && w.meta >= 0;
       if (active) {
-        const int nh_new = 255 - int(my_key >> 56);
-        const float chi2_new = __uint_as_float(uint32_t(my_key >> 24));
-        const int hit_plus1 = int(my_key & 0x1fffffu);
+        int hit = -1;
         int32_t st_new = pst;
-        if (hit_plus1 > 0) {
-          const float4 m = B.hits[h0 + my_pos];
+        if (w.pos >= 0) {
+          const float4 m = B.hits[h0 + w.pos];
+          hit = __float_as_int(m.w);
           float r0, r1, r2;
           kf::residual<float, true>(q, ql, m.x, m.y, m.z, r0, r1, r2);
           kf::kalman_update<float, true>(q, ql, qC, qS, r0, r1, r2, A.v0, A.v1, A.v2);
@@ -1165,16 +1292,16 @@ __global__ void __launch_bounds__(kResThreads, resident_blocks_per_sm(W))
           st_new |= KF_ST_NO_HIT;
         }
         const int64_t hslot = int64_t(l) * S8 + cand_slot(j, k, B.S, l + 1 < A.rm_buffers);
-        B.hist_parent[hslot] = int8_t((my_key >> 21) & 7u);
-        B.hist_hit[hslot] = hit_plus1 - 1;
+        B.hist_parent[hslot] = int8_t(w.meta & 7);
+        B.hist_hit[hslot] = hit;
 #pragma unroll
         for (int c = 0; c < 6; ++c) p[c] = q[c];
 #pragma unroll
         for (int c = 0; c < 3; ++c) lo[c] = ql[c];
 #pragma unroll
         for (int c = 0; c < 21; ++c) C[c] = qC[c];
-        chi2tot = chi2_new;
-        nh = nh_new;
+        chi2tot = __uint_as_float(w.x);
+        nh = w.meta >> 8;
         st = st_new;
       }
     }
@@ -1249,6 +1376,7 @@ __global__ void __launch_bounds__(kResThreads, resident_blocks_per_sm(W))
 template <bool TABLE, bool MAT>
 __global__ void __launch_bounds__(kResThreads, kResBlocksPerSM)
     build_first_layer_kernel(const __grid_constant__ BuildResidentArgs A) {
+  __shared__ float4 s_stage[kScanStage * kResThreads];
   const int64_t t = int64_t(blockIdx.x) * kResThreads + threadIdx.x;
   int q = 0;  // the batch of this seed (a served event), with a table
   if constexpr (TABLE) {
@@ -1291,7 +1419,7 @@ __global__ void __launch_bounds__(kResThreads, kResBlocksPerSM)
   const int64_t h0 = B.seg_off[sg];
   bool stopped = (st & KF_ST_STOPPED) != 0;
   if (!stopped) {
-    const int r = kf::propagate<float, kNewtonBuild, true>(p, lo, C, a, A.R[l]);
+    const int r = kf::propagate<float, kNewtonBuild, true, true>(p, lo, C, a, A.R[l]);
     if (r) {
       st |= r;
       stopped = true;
@@ -1300,35 +1428,39 @@ __global__ void __launch_bounds__(kResThreads, kResBlocksPerSM)
     }
   }
   float Si[6] = {0.f, 0.f, 0.f, 0.f, 0.f, 0.f};
-  uint64_t L[kGroup];
+  uint32_t X[kGroup];
   int P[kGroup];
 #pragma unroll
   for (int t = 0; t < kGroup; ++t) {
-    L[t] = kNoKey;
+    X[t] = kNoChild;
     P[t] = -1;
   }
-  bool any = false;
   if (!stopped) {
     const int nphi = B.fine_off ? KF_BIN_PHI_FINE : KF_BIN_PHI;
     const int32_t* boff = B.fine_off ? B.fine_off + sg * (KF_NBINS_FINE + 1) : B.bin_off + sg * (KF_NBINS + 1);
     int e0 = 0, e1 = -1, fa0 = 0, fa1 = nphi - 1, fb0 = 0, fb1 = -1;
-    hit_window(p, lo, C, A.R[l], A.v0, A.v1, A.v2, A.cut, Si, e0, e1, fa0, fa1, fb0, fb1, nphi);
-    any = scan_window(p, lo, Si, e0, e1, fa0, fa1, fb0, fb1, boff, B.hits + h0, A.cut, nh, chi2tot, 0, L, P, nphi);
+    hit_window(p, lo, C, A.R[l], A.v0, A.v1, A.v2, A.cut, e0, e1, fa0, fa1, fb0, fb1, nphi);
+    scan_children(p, lo, C, A.v0, A.v1, A.v2, Si, e0, e1, fa0, fa1, fb0, fb1, boff, B.hits + h0, A.cut, chi2tot, X, P,
+                  nphi, s_stage + threadIdx.x);
   }
   // no compatible hit (or a stopped seed): one child without a hit
-  if (!any) list_insert(L, P, make_key(nh, chi2tot, 0, 0), -1);
+  int nhk = nh + 1;
+  if (X[0] == kNoChild) {
+    X[0] = __float_as_uint(chi2tot);
+    nhk = nh;
+  }
   int n_win = 0;
 #pragma unroll 1
   for (int r = 0; r < A.max_cands; ++r) {
-    uint64_t key = kNoKey;
+    uint32_t x = kNoChild;
     int pos = -1;
 #pragma unroll
     for (int t = 0; t < kGroup; ++t)
       if (t == r) {
-        key = L[t];
+        x = X[t];
         pos = P[t];
       }
-    if (key == kNoKey) break;
+    if (x == kNoChild) break;
     ++n_win;
     float q[6], ql[3], qC[21];
 #pragma unroll
@@ -1337,12 +1469,11 @@ __global__ void __launch_bounds__(kResThreads, kResBlocksPerSM)
     for (int c = 0; c < 3; ++c) ql[c] = lo[c];
 #pragma unroll
     for (int c = 0; c < 21; ++c) qC[c] = C[c];
-    const int nh_new = 255 - int(key >> 56);
-    const float chi2_new = __uint_as_float(uint32_t(key >> 24));
-    const int hit_plus1 = int(key & 0x1fffffu);
+    int hit = -1;
     int32_t st_new = st;
-    if (hit_plus1 > 0) {
+    if (pos >= 0) {
       const float4 m = B.hits[h0 + pos];
+      hit = __float_as_int(m.w);
       float r0, r1, r2;
       kf::residual<float, true>(q, ql, m.x, m.y, m.z, r0, r1, r2);
       kf::kalman_update<float, true>(q, ql, qC, Si, r0, r1, r2, A.v0, A.v1, A.v2);
@@ -1356,10 +1487,10 @@ __global__ void __launch_bounds__(kResThreads, kResBlocksPerSM)
     for (int c = 0; c < 3; ++c) B.out.par[(6 + c) * S8 + os] = ql[c];
 #pragma unroll
     for (int c = 0; c < 21; ++c) B.out.cov[c * S8 + os] = qC[c];
-    B.out.chi2[os] = chi2_new;
-    B.out.meta[os] = nh_new | (st_new << 8);
+    B.out.chi2[os] = __uint_as_float(x);
+    B.out.meta[os] = nhk | (st_new << 8);
     B.hist_parent[int64_t(l) * S8 + os] = 0;
-    B.hist_hit[int64_t(l) * S8 + os] = hit_plus1 - 1;
+    B.hist_hit[int64_t(l) * S8 + os] = hit;
   }
   B.out.ncand[j] = int8_t(n_win);
 }
