@@ -3,12 +3,13 @@
 // phi within eta bins, phi bins for fast look-up of compatible hits).
 //
 // A counting sort of every segment (one event on one layer) into the 64 x 256
-// bins, with a final insertion sort by id inside each bin so that the output
-// is deterministic (skipped with kf_tuning.bin_unordered: the build's results
-// do not depend on the order of the hits inside a bin).  The unordered form
-// can sort by 64 x 512 sub-bins instead, each bin two of them, and give the
-// sub-bin starts as well: the build's windows then cover half as wide a
-// strip of phi beyond their edges.
+// bins, either by passes over all points of all segments at once or by one
+// block per segment (launch_bin_points), with a final pass that orders each
+// bin by id so that the output is deterministic (skipped with
+// kf_tuning.bin_unordered: the build's results do not depend on the order of
+// the hits inside a bin).  The unordered form can sort by 64 x 512 sub-bins
+// instead, each bin two of them, and give the sub-bin starts as well: the
+// build's windows then cover half as wide a strip of phi beyond their edges.
 #include "kf_bin.cuh"
 #include "kf_internal.h"
 
@@ -17,40 +18,9 @@
 
 namespace kfi {
 
-// The ordered binning: a counting sort over all points of all segments at
-// once, in four fully parallel passes: (1) every point adds one to its segment's count of its
-// bin (global atomics into bin_off), (2) one block per segment turns the
-// counts into exclusive offsets (bin_off) and scatter cursors, (3) every
-// point takes the next slot of its bin, (4) one thread per (segment, bin)
-// sorts the bin's slots by id, so the output does not depend on the order
-// in which (3) took them.  A segment of any size spreads over the whole GPU.
 constexpr int kScanThreads = 1024;
 static_assert(KF_NBINS % kScanThreads == 0, "bins per thread");  // 16 consecutive bins a thread
 constexpr int kPointThreads = 256;
-
-// the segment s with seg_off[s] <= g < seg_off[s + 1], or -1
-__device__ __forceinline__ int segment_of(const int64_t* off, int nseg, int64_t g) {
-  if (g < off[0] || g >= off[nseg]) return -1;
-  int lo = 0, hi = nseg - 1;
-  while (lo < hi) {
-    const int mid = (lo + hi + 1) >> 1;
-    if (off[mid] <= g)
-      lo = mid;
-    else
-      hi = mid - 1;
-  }
-  return g < off[lo + 1] ? lo : -1;
-}
-
-__global__ void __launch_bounds__(kPointThreads) bin_count_kernel(const BinArgs A, int nseg) {
-  const int64_t stride = int64_t(gridDim.x) * blockDim.x;
-  for (int64_t g = int64_t(blockIdx.x) * blockDim.x + threadIdx.x; g < A.stride; g += stride) {
-    const int s = segment_of(A.seg_off, nseg, g);
-    if (s < 0) continue;
-    const int b = bin_of(A.xyz[g], A.xyz[A.stride + g], A.xyz[2 * A.stride + g]);
-    atomicAdd(&A.bin_off[int64_t(s) * (KF_NBINS + 1) + b], 1);
-  }
-}
 
 // padded shared-memory index of bin b: a thread's 16 (or 32) consecutive
 // bins and a warp's 32 threads fall in distinct banks
@@ -100,24 +70,6 @@ __device__ __forceinline__ int scan_bins(int* cnt, int* warp_tot) {
   }
   __syncthreads();
   return total;
-}
-
-__global__ void __launch_bounds__(kScanThreads) bin_scan_kernel(const BinArgs A) {
-  extern __shared__ int cnt[];  // counts, then offsets (padded layout)
-  __shared__ int warp_tot[32];
-  const int seg = blockIdx.x;
-  int32_t* off = A.bin_off + int64_t(seg) * (KF_NBINS + 1);
-  int32_t* cur = A.cursor + int64_t(seg) * KF_NBINS;
-  const int tid = threadIdx.x;
-  for (int b = tid; b < KF_NBINS; b += kScanThreads) cnt[pad_idx(b)] = off[b];  // coalesced
-  __syncthreads();
-  const int total = scan_bins(cnt, warp_tot);
-  if (tid == 0) off[KF_NBINS] = total;
-  for (int b = tid; b < KF_NBINS; b += kScanThreads) {  // coalesced
-    const int o = cnt[pad_idx(b)];
-    off[b] = o;
-    cur[b] = o;
-  }
 }
 
 // The unordered counting sort of one segment per block, its counts and
@@ -221,54 +173,194 @@ __global__ void __launch_bounds__(kScanThreads) bin_segment_kernel(const BinArgs
                         A.out_seg, seg, cnt, warp_tot);
 }
 
-// The same over a table of segments of different point sets (the events a
-// serving iteration prepares), one block per entry.
+// ---------------------------------------------------------------------------
+// The passes over all points of all segments at once: a segment of any size
+// spreads over the whole GPU.
+//   (zero)            the counts, in the bin (or sub-bin) starts' own place
+//   bin_count_kernel  every point adds one to its bin's count; the count before
+//                     it is its place in the bin, kept with the bin in one word
+//   bin_scan_kernel   one block per segment: counts to starts
+//   bin_place_kernel  every point to its bin's start plus its place
+//   bin_order_kernel  (ordered form) a warp sorts the hits of 32 consecutive
+//                     bins, a contiguous run, by id inside each bin
+// A point's word between the passes: its bin above its place, or, with the top
+// bit set, its position in the segment.  A place of kPlaceMax or more (a bin of
+// more than 65 535 hits) does not fit: the count leaves it in the point's own
+// entry of the output, and the scan, between the two passes, turns it into a
+// position.
+constexpr int kPlaceBits = 16;
+constexpr uint32_t kPlaceMax = (1u << kPlaceBits) - 1;
+constexpr uint32_t kIsPosition = 1u << 31;
+static_assert(KF_NBINS_FINE <= 1 << (31 - kPlaceBits), "bin and place in a word");
+
+// segment s of the request: a table entry, or segment s of the arrays of A
 template <bool FINE>
-__global__ void __launch_bounds__(kScanThreads) bin_segment_table_kernel(const BinSegment* table) {
-  extern __shared__ int cnt[];
-  __shared__ int warp_tot[32];
-  const BinSegment& T = table[blockIdx.x];
-  bin_one_segment<FINE>(T.xyz, T.stride, T.p0, T.p1, T.bin_off, T.fine_off, T.out_pts, T.out_id, nullptr, 0, cnt,
-                        warp_tot);
+__device__ __forceinline__ BinSegment segment(const BinArgs& A, int s) {
+  if (A.table) return A.table[s];
+  BinSegment S;
+  S.xyz = A.xyz;
+  S.stride = A.stride;
+  S.p0 = A.seg_off[s];
+  S.p1 = min(A.seg_off[s + 1], A.stride);
+  S.begin = S.p0;
+  S.bin_off = A.bin_off + int64_t(s) * (KF_NBINS + 1);
+  S.fine_off = FINE ? A.fine_off + int64_t(s) * (KF_NBINS_FINE + 1) : nullptr;
+  S.out_pts = A.out_pts;
+  S.out_id = A.out_id;
+  return S;
 }
-
-__global__ void __launch_bounds__(kPointThreads) bin_scatter_kernel(const BinArgs A, int nseg) {
-  const int64_t stride = int64_t(gridDim.x) * blockDim.x;
-  for (int64_t g = int64_t(blockIdx.x) * blockDim.x + threadIdx.x; g < A.stride; g += stride) {
-    const int s = segment_of(A.seg_off, nseg, g);
-    if (s < 0) continue;
-    const float x = A.xyz[g], y = A.xyz[A.stride + g], z = A.xyz[2 * A.stride + g];
-    const int b = bin_of(x, y, z);
-    const int64_t p0 = A.seg_off[s];
-    const int i = int(g - p0);
-    const int64_t q = p0 + atomicAdd(&A.cursor[int64_t(s) * KF_NBINS + b], 1);
-    if (q >= A.stride) continue;  // only for malformed offsets
-    A.out_id[q] = i;
-    if (A.out_pts) A.out_pts[q] = make_float4(x, y, z, __int_as_float(i));
-    if (A.out_seg) A.out_seg[q] = s;
+// the last segment that begins at or before point g of the launch's points
+__device__ __forceinline__ int segment_of(const BinArgs& A, int64_t g) {
+  int lo = 0, hi = A.n_seg - 1;
+  while (lo < hi) {
+    const int mid = (lo + hi + 1) >> 1;
+    if ((A.table ? A.table[mid].begin : A.seg_off[mid]) <= g)
+      lo = mid;
+    else
+      hi = mid - 1;
   }
+  return lo;
 }
 
-// deterministic order: insertion sort by id inside each bin
-__global__ void __launch_bounds__(kPointThreads) bin_sort_kernel(const BinArgs A, int nseg) {
-  const int64_t t = int64_t(blockIdx.x) * blockDim.x + threadIdx.x;
-  if (t >= int64_t(nseg) * KF_NBINS) return;
-  const int s = int(t / KF_NBINS), b = int(t % KF_NBINS);
-  const int32_t* off = A.bin_off + int64_t(s) * (KF_NBINS + 1);
-  const int64_t p0 = A.seg_off[s];
-  int64_t beg = p0 + off[b], end = p0 + off[b + 1];
-  if (end > A.stride) end = A.stride;
-  for (int64_t u = beg + 1; u < end; ++u) {
-    const int id = A.out_id[u];
-    const float4 pt = A.out_pts ? A.out_pts[u] : make_float4(0.f, 0.f, 0.f, 0.f);
-    int64_t v = u - 1;
-    while (v >= beg && A.out_id[v] > id) {
-      A.out_id[v + 1] = A.out_id[v];
-      if (A.out_pts) A.out_pts[v + 1] = A.out_pts[v];
-      --v;
+template <bool FINE>
+__global__ void __launch_bounds__(kPointThreads) bin_zero_kernel(const BinArgs A) {
+  const BinSegment S = segment<FINE>(A, int(blockIdx.y));
+  (FINE ? S.fine_off : S.bin_off)[blockIdx.x * kPointThreads + threadIdx.x] = 0;
+}
+
+template <bool FINE>
+__global__ void __launch_bounds__(kPointThreads) bin_count_kernel(const BinArgs A) {
+  const int64_t g = int64_t(blockIdx.x) * kPointThreads + threadIdx.x;
+  if (g >= A.n_points) return;
+  const BinSegment S = segment<FINE>(A, segment_of(A, g));
+  const int64_t q = g - S.begin + S.p0;
+  if (q < S.p0 || q >= S.p1) return;  // outside every segment
+  const int b = bin_of<FINE ? KF_BIN_PHI_FINE : KF_BIN_PHI>(S.xyz[q], S.xyz[S.stride + q], S.xyz[2 * S.stride + q]);
+  const uint32_t place = uint32_t(atomicAdd((FINE ? S.fine_off : S.bin_off) + b, 1));
+  if (place >= kPlaceMax) S.out_pts[q].x = __uint_as_float(place);
+  S.out_id[q] = int(uint32_t(b) << kPlaceBits | min(place, kPlaceMax));
+}
+
+template <bool FINE>
+__global__ void __launch_bounds__(kScanThreads) bin_scan_kernel(const BinArgs A) {
+  constexpr int NB = FINE ? KF_NBINS_FINE : KF_NBINS;
+  constexpr int kPer = NB / kScanThreads;
+  extern __shared__ int cnt[];  // counts, then starts (padded layout)
+  __shared__ int warp_tot[32];
+  const BinSegment S = segment<FINE>(A, int(blockIdx.x));
+  int32_t* const c = FINE ? S.fine_off : S.bin_off;
+  const int tid = threadIdx.x;
+  // 16 loads a thread in flight together (coalesced): one after the other they
+  // were two thirds of the pass when few segments leave most SMs idle
+  bool over = false;  // a bin with places that do not fit their words
+#pragma unroll 1
+  for (int t0 = 0; t0 < kPer; t0 += 16) {
+    int v[16];
+#pragma unroll
+    for (int t = 0; t < 16; ++t) v[t] = c[(t0 + t) * kScanThreads + tid];
+#pragma unroll
+    for (int t = 0; t < 16; ++t) {
+      cnt[pad_idx((t0 + t) * kScanThreads + tid)] = v[t];
+      over |= v[t] > int(kPlaceMax);
     }
-    A.out_id[v + 1] = id;
-    if (A.out_pts) A.out_pts[v + 1] = pt;
+  }
+  over = __syncthreads_or(over);
+  const int total = scan_bins<NB>(cnt, warp_tot);
+  if (tid == 0) c[NB] = total;
+  for (int b = tid; b < NB; b += kScanThreads) c[b] = cnt[pad_idx(b)];
+  if constexpr (FINE) {
+    if (tid == 0) S.bin_off[KF_NBINS] = total;
+    for (int b = tid; b < KF_NBINS; b += kScanThreads) S.bin_off[b] = cnt[pad_idx(2 * b)];
+  }
+  if (over)
+    for (int64_t q = S.p0 + tid; q < S.p1; q += kScanThreads) {
+      const uint32_t w = uint32_t(S.out_id[q]);
+      if ((w & kPlaceMax) == kPlaceMax)
+        S.out_id[q] = int(kIsPosition | (uint32_t(cnt[pad_idx(int(w >> kPlaceBits))]) + __float_as_uint(S.out_pts[q].x)));
+    }
+}
+
+template <bool FINE>
+__global__ void __launch_bounds__(kPointThreads) bin_place_kernel(const BinArgs A) {
+  const int64_t g = int64_t(blockIdx.x) * kPointThreads + threadIdx.x;
+  if (g >= A.n_points) return;
+  const BinSegment S = segment<FINE>(A, segment_of(A, g));
+  const int64_t q = g - S.begin + S.p0;
+  if (q < S.p0 || q >= S.p1) return;
+  const float x = S.xyz[q], y = S.xyz[S.stride + q], z = S.xyz[2 * S.stride + q];
+  const uint32_t w = uint32_t(S.out_id[q]);
+  const int at = w & kIsPosition ? int(w & ~kIsPosition)
+                                 : (FINE ? S.fine_off : S.bin_off)[w >> kPlaceBits] + int(w & kPlaceMax);
+  S.out_pts[S.p0 + at] = make_float4(x, y, z, __int_as_float(int(q - S.p0)));
+}
+
+// One warp per 32 bins of a segment: their hits, ids in any order inside a
+// bin, are a contiguous run.  Runs of up to kOrderRun hits are taken whole:
+// loaded (coalesced, all in flight), every hit's place found by counting the
+// smaller ids of its bin in shared memory, and the moved ones written back.
+// Of a longer run, as many bins as fit are taken at a time; a single bin that
+// does not fit is sorted by one insertion sort.
+constexpr int kOrderRun = 128;
+constexpr int kOrderWarps = 4;
+__global__ void __launch_bounds__(32 * kOrderWarps) bin_order_kernel(const BinArgs A) {
+  __shared__ int s_id[kOrderWarps][kOrderRun];
+  __shared__ int s_off[kOrderWarps][33];
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  int* const ids = s_id[warp];
+  int* const off = s_off[warp];
+  const int s = int(blockIdx.x) / (KF_NBINS / 32 / kOrderWarps);
+  const int b0 = (int(blockIdx.x) % (KF_NBINS / 32 / kOrderWarps) * kOrderWarps + warp) * 32;
+  const int32_t* const starts = A.bin_off + int64_t(s) * (KF_NBINS + 1) + b0;
+  float4* const pts = A.out_pts + A.seg_off[s];
+  const int mine = starts[lane];
+  off[lane] = mine;
+  if (lane == 0) off[32] = starts[32];
+  __syncwarp();
+  const int end_all = off[32];
+  for (int bb = 0; bb < 32 && off[bb] < end_all;) {
+    const int beg = off[bb];
+    // the bins bb .. be-1 whose hits fit a run
+    int be = 33 - __popc(__ballot_sync(0xffffffffu, off[lane + 1] - beg > kOrderRun && lane >= bb)) - 1;
+    if (be == bb) {  // one bin alone is too long
+      if (lane == 0)
+        for (int u = beg + 1; u < off[bb + 1]; ++u) {
+          const float4 pt = pts[u];
+          int v = u - 1;
+          for (; v >= beg && __float_as_int(pts[v].w) > __float_as_int(pt.w); --v) pts[v + 1] = pts[v];
+          pts[v + 1] = pt;
+        }
+      bb = be + 1;
+      continue;
+    }
+    const int n = off[be] - beg;
+    float4 h[kOrderRun / 32];
+#pragma unroll
+    for (int t = 0; t < kOrderRun / 32; ++t)
+      if (lane + 32 * t < n) h[t] = pts[beg + lane + 32 * t];
+#pragma unroll
+    for (int t = 0; t < kOrderRun / 32; ++t)
+      if (lane + 32 * t < n) ids[lane + 32 * t] = __float_as_int(h[t].w);
+    __syncwarp();
+#pragma unroll
+    for (int t = 0; t < kOrderRun / 32; ++t) {
+      const int i = lane + 32 * t;
+      if (i < n) {
+        int lo = bb, hi = be - 1;  // the bin of hit i
+        while (lo < hi) {
+          const int mid = (lo + hi + 1) >> 1;
+          if (off[mid] - beg <= i)
+            lo = mid;
+          else
+            hi = mid - 1;
+        }
+        const int first = off[lo] - beg, last = off[lo + 1] - beg, id = ids[i];
+        int at = first;
+        for (int u = first; u < last; ++u) at += ids[u] < id ? 1 : 0;
+        if (at != i) pts[beg + at] = h[t];
+      }
+    }
+    __syncwarp();  // ids are read before the next run's
+    bb = be;
   }
 }
 
@@ -293,60 +385,65 @@ static cudaError_t segment_smem_attrs(K kernel, int smem, std::atomic<bool>* don
   return e;
 }
 
-cudaError_t launch_bin_segment_table(const BinSegment* table, int n, bool fine, cudaStream_t st) {
-  if (n <= 0) return cudaSuccess;
-  static std::atomic<bool> attr_set[kMaxDevices], fine_attr_set[kMaxDevices];
-  if (fine) {
-    cudaError_t e = segment_smem_attrs(bin_segment_table_kernel<true>, kFineSmem, fine_attr_set);
-    if (e != cudaSuccess) return e;
-    bin_segment_table_kernel<true><<<n, kScanThreads, kFineSmem, st>>>(table);
-    return cudaGetLastError();
-  }
-  cudaError_t e = segment_smem_attrs(bin_segment_table_kernel<false>, kScanSmem, attr_set);
+template <bool FINE>
+static cudaError_t launch_bin_wide(const BinArgs& a, cudaStream_t st) {
+  static std::atomic<bool> attr_set[kMaxDevices];
+  constexpr int smem = FINE ? kFineSmem : kScanSmem;
+  cudaError_t e = segment_smem_attrs(bin_scan_kernel<FINE>, smem, attr_set);
   if (e != cudaSuccess) return e;
-  bin_segment_table_kernel<false><<<n, kScanThreads, kScanSmem, st>>>(table);
+  if (a.table)
+    bin_zero_kernel<FINE><<<dim3((FINE ? KF_NBINS_FINE : KF_NBINS) / kPointThreads, a.n_seg), kPointThreads, 0, st>>>(a);
+  else
+    e = cudaMemsetAsync(FINE ? a.fine_off : a.bin_off, 0,
+                        size_t(a.n_seg) * ((FINE ? KF_NBINS_FINE : KF_NBINS) + 1) * sizeof(int32_t), st);
+  if (e != cudaSuccess) return e;
+  const unsigned grid = unsigned((a.n_points + kPointThreads - 1) / kPointThreads);
+  if (grid > 0) bin_count_kernel<FINE><<<grid, kPointThreads, 0, st>>>(a);
+  bin_scan_kernel<FINE><<<a.n_seg, kScanThreads, smem, st>>>(a);
+  if (grid > 0) bin_place_kernel<FINE><<<grid, kPointThreads, 0, st>>>(a);
   return cudaGetLastError();
 }
 
-cudaError_t launch_bin_points(const BinArgs& a, int n_segments, cudaStream_t st) {
-  if (n_segments <= 0) return cudaSuccess;
-  int dev = 0;
-  cudaError_t e = cudaGetDevice(&dev);
-  if (e != cudaSuccess) return e;
-  if (a.unordered) {  // one launch, one block per segment
+cudaError_t launch_bin_segment_table(const BinSegment* table, int n, int64_t n_points, bool fine, cudaStream_t st) {
+  if (n <= 0) return cudaSuccess;
+  BinArgs a;
+  a.table = table;
+  a.n_seg = n;
+  a.n_points = n_points;
+  return fine ? launch_bin_wide<true>(a, st) : launch_bin_wide<false>(a, st);
+}
+
+// Which form: one block per segment costs about 10 us plus 1.3 us per 1 000
+// hits of the largest segment, times the rounds of segments on the SMs; the
+// wide passes 20 us plus 0.024 us per 1 000 hits of all segments (measured:
+// 350 segments of 20 000 hits 158 against 185 us, by sub-bin 182 against 210;
+// 28 of 3 000: 18 against 24; 7 of 20 000: 35 against 24; 7 of 200 000: 285
+// against 48; 84 uneven ones of 23 000 on average: 132 against 66).  The sizes
+// are on the device, so the rule goes by their mean: blocks for many segments,
+// among which a large one weighs little, and for small ones.
+static bool one_block_a_segment(const BinArgs& a, int num_sms) {
+  return !a.out_pts || a.n_points <= int64_t(a.n_seg) * (a.n_seg >= num_sms ? 40000 : 3000);
+}
+
+cudaError_t launch_bin_points(const BinArgs& a, int num_sms, cudaStream_t st) {
+  if (a.n_seg <= 0) return cudaSuccess;
+  if (a.fine_off && !a.unordered) return cudaErrorInvalidValue;  // sub-bins only with the unordered binning
+  cudaError_t e;
+  if (!one_block_a_segment(a, num_sms)) {
+    e = a.fine_off ? launch_bin_wide<true>(a, st) : launch_bin_wide<false>(a, st);
+  } else {
     static std::atomic<bool> seg_attr_set[kMaxDevices], fine_attr_set[kMaxDevices];
     if (a.fine_off) {
       e = segment_smem_attrs(bin_segment_kernel<true>, kFineSmem, fine_attr_set);
-      if (e != cudaSuccess) return e;
-      bin_segment_kernel<true><<<n_segments, kScanThreads, kFineSmem, st>>>(a);
-      return cudaGetLastError();
+      if (e == cudaSuccess) bin_segment_kernel<true><<<a.n_seg, kScanThreads, kFineSmem, st>>>(a);
+    } else {
+      e = segment_smem_attrs(bin_segment_kernel<false>, kScanSmem, seg_attr_set);
+      if (e == cudaSuccess) bin_segment_kernel<false><<<a.n_seg, kScanThreads, kScanSmem, st>>>(a);
     }
-    e = segment_smem_attrs(bin_segment_kernel<false>, kScanSmem, seg_attr_set);
-    if (e != cudaSuccess) return e;
-    bin_segment_kernel<false><<<n_segments, kScanThreads, kScanSmem, st>>>(a);
-    return cudaGetLastError();
   }
-  if (a.fine_off) return cudaErrorInvalidValue;  // sub-bins only with the unordered binning
-  e = cudaMemsetAsync(a.bin_off, 0, size_t(n_segments) * (KF_NBINS + 1) * sizeof(int32_t), st);
-  if (e != cudaSuccess) return e;
-  const int64_t pts = a.stride > 0 ? a.stride : 1;
-  const int pgrid = int(std::min<int64_t>((pts + kPointThreads - 1) / kPointThreads, int64_t(1) << 20));
-  bin_count_kernel<<<pgrid, kPointThreads, 0, st>>>(a, n_segments);
-  // the scan kernel's shared-memory attribute, set once per device (the
-  // serving loop bins point sets of many events; setting it again from
-  // another thread is harmless, the value being the same)
-  static std::atomic<bool> scan_attr_set[kMaxDevices];
-  if (dev < 0 || dev >= kMaxDevices || !scan_attr_set[dev].load(std::memory_order_acquire)) {
-    e = cudaFuncSetAttribute(bin_scan_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, kScanSmem);
-    if (e != cudaSuccess) return e;
-    if (dev >= 0 && dev < kMaxDevices) scan_attr_set[dev].store(true, std::memory_order_release);
-  }
-  bin_scan_kernel<<<n_segments, kScanThreads, kScanSmem, st>>>(a);
-  bin_scatter_kernel<<<pgrid, kPointThreads, 0, st>>>(a, n_segments);
-  const int64_t bins = int64_t(n_segments) * KF_NBINS;
-  if (!a.unordered)
-    bin_sort_kernel<<<int((bins + kPointThreads - 1) / kPointThreads), kPointThreads, 0, st>>>(a, n_segments);
-  return cudaGetLastError();
+  if (e == cudaSuccess && !a.unordered && a.n_points > 0)
+    bin_order_kernel<<<unsigned(a.n_seg) * (KF_NBINS / 32 / kOrderWarps), 32 * kOrderWarps, 0, st>>>(a);
+  return e != cudaSuccess ? e : cudaGetLastError();
 }
 
 }  // namespace kfi
@@ -369,19 +466,20 @@ extern "C" int kf_bin_hits(kf_ctx* ctx, const kf_layer_hits* in, kf_layer_hit_bi
   if (nseg == 0) return KF_OK;
   KF_CUDA_TRY(ctx, cudaSetDevice(ctx->device));
   const size_t id_bytes = (size_t(in->n_hits > 0 ? in->n_hits : 1) * sizeof(int32_t) + 255) & ~size_t(255);
-  int rc = scratch_reserve(ctx, ctx->s_bin_id, id_bytes + size_t(nseg) * KF_NBINS * sizeof(int32_t));
+  int rc = scratch_reserve(ctx, ctx->s_bin_id, id_bytes);
   if (rc) return rc;
   BinArgs a;
   a.xyz = in->xyz;
   a.stride = in->n_hits;
   a.seg_off = in->seg_off;
+  a.n_seg = nseg;
+  a.n_points = in->n_hits;
   a.bin_off = out->bin_off;
   a.out_pts = reinterpret_cast<float4*>(out->hits);
   a.out_id = static_cast<int32_t*>(ctx->s_bin_id.ptr);
   a.out_seg = nullptr;
-  a.cursor = reinterpret_cast<int32_t*>(static_cast<char*>(ctx->s_bin_id.ptr) + id_bytes);
   a.unordered = ctx->tune.bin_unordered;
   a.fine_off = out->fine_off;
-  KF_CUDA_TRY(ctx, launch_bin_points(a, nseg, static_cast<cudaStream_t>(stream)));
+  KF_CUDA_TRY(ctx, launch_bin_points(a, ctx->num_sms, static_cast<cudaStream_t>(stream)));
   return KF_OK;
 }

@@ -36,21 +36,6 @@ __device__ __forceinline__ int bin_of(float x, float y, float z) {
   return eta_bin(eta) * NPHI + phi_bin_n<NPHI>(atan2f(y, x));
 }
 
-struct BinArgs {
-  const float* xyz;        // [3][stride]
-  int64_t stride;
-  const int64_t* seg_off;  // [n_seg + 1]
-  int32_t* bin_off;        // [n_seg][KF_NBINS + 1] required: bin starts within the segment, then the count
-  float4* out_pts;         // [total] or null
-  int32_t* out_id;         // [total] required: id within the segment, bin order (unordered, with
-                           // out_pts: scratch, left holding each point's bin in input order)
-  int32_t* out_seg;        // [total] or null
-  int32_t* cursor;         // [n_seg][KF_NBINS] scratch
-  int unordered = 0;       // 1: leave each bin in scatter order (no sort by id)
-  int32_t* fine_off = nullptr;  // unordered only: [n_seg][KF_NBINS_FINE + 1] sub-bin starts, or null;
-                                // when set the points are ordered by sub-bin
-};
-
 // One segment of a table-driven unordered binning: points [p0, p1) of xyz
 // ([3][stride]), their offsets into bin_off ([KF_NBINS + 1]) and, with the
 // sub-bins, fine_off ([KF_NBINS_FINE + 1]), points into out_pts[p0 .. p1),
@@ -59,18 +44,36 @@ struct BinSegment {
   const float* xyz;
   int64_t stride;
   int64_t p0, p1;
+  int64_t begin;  // its first point in the numbering of all points of the table
   int32_t* bin_off;
   int32_t* fine_off;
   float4* out_pts;
   int32_t* out_id;
 };
-// Bin the n segments of a device table in one launch (unordered; fine: by
-// sub-bin, every entry's fine_off set).
-cudaError_t launch_bin_segment_table(const BinSegment* table, int n, bool fine, cudaStream_t st);
 
-// Sort the points of every segment into bins (several launches on `st`);
-// stride is the number of points (the segments cover [seg_off[0],
-// seg_off[n_segments])).
-cudaError_t launch_bin_points(const BinArgs& a, int n_segments, cudaStream_t st);
+struct BinArgs {
+  const float* xyz = nullptr;         // [3][stride]
+  int64_t stride = 0;
+  const int64_t* seg_off = nullptr;   // [n_seg + 1]
+  const BinSegment* table = nullptr;  // [n_seg] segments of different point sets, in place of the arrays here
+  int n_seg = 0;
+  int64_t n_points = 0;               // of all segments (with the arrays: stride)
+  int32_t* bin_off = nullptr;         // [n_seg][KF_NBINS + 1] required: bin starts within the segment, then the count
+  float4* out_pts = nullptr;          // [total] or null
+  int32_t* out_id = nullptr;          // [total] required: id within the segment, bin order (with
+                                      // out_pts: scratch, each point's bin and place in input order)
+  int32_t* out_seg = nullptr;         // [total] or null
+  int unordered = 0;                  // 1: leave each bin in scatter order (no sort by id)
+  int32_t* fine_off = nullptr;        // unordered only: [n_seg][KF_NBINS_FINE + 1] sub-bin starts, or null;
+                                      // when set the points are ordered by sub-bin
+};
+
+// Bin the n segments of a device table, n_points points in all (unordered;
+// fine: by sub-bin, every entry's fine_off set).
+cudaError_t launch_bin_segment_table(const BinSegment* table, int n, int64_t n_points, bool fine, cudaStream_t st);
+
+// Sort the points of every segment of `a` into bins (one or several launches on
+// `st`).  out_pts null (seeds): the ids only, unordered, one block per segment.
+cudaError_t launch_bin_points(const BinArgs& a, int num_sms, cudaStream_t st);
 
 }  // namespace kfi

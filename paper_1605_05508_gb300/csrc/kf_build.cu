@@ -1736,9 +1736,9 @@ extern "C" int kf_build(kf_ctx* ctx, const kf_tracks* seeds, const int64_t* seed
   const size_t b_hp = al256(size_t(L) * S8), b_hh = al256(size_t(L) * S8 * 4);
   const size_t b_tab = al256(sizeof(BuildSlot) * size_t(L));
   const int64_t E = bins->n_events;
-  const size_t b_sbin = al256(size_t(E) * (KF_NBINS + 1) * 4), b_scur = al256(size_t(E) * KF_NBINS * 4);
+  const size_t b_sbin = al256(size_t(E) * (KF_NBINS + 1) * 4);
   const size_t b_ctr = 256;  // the resident build's group counter
-  const size_t total = b_perm + b_evt + 2 * b_cand + b_hp + b_hh + b_tab + b_sbin + b_scur + b_ctr;
+  const size_t total = b_perm + b_evt + 2 * b_cand + b_hp + b_hh + b_tab + b_sbin + b_ctr;
   int rc = scratch_reserve(ctx, ctx->s_build, total);
   if (rc) return rc;
   char* base = static_cast<char*>(ctx->s_build.ptr);
@@ -1764,15 +1764,16 @@ extern "C" int kf_build(kf_ctx* ctx, const kf_tracks* seeds, const int64_t* seed
   BinArgs ba;
   ba.xyz = seeds->par;
   ba.stride = S;
+  ba.n_seg = bins->n_events;
+  ba.n_points = S;
   ba.seg_off = seed_off;
   ba.bin_off = reinterpret_cast<int32_t*>(base + b_perm + b_evt + 2 * b_cand + b_hp + b_hh + b_tab);
   ba.out_pts = nullptr;
   ba.out_id = perm;
   ba.out_seg = evt;
-  ba.cursor = reinterpret_cast<int32_t*>(base + b_perm + b_evt + 2 * b_cand + b_hp + b_hh + b_tab + b_sbin);
   ba.unordered = 1;  // each seed's result is independent of the order of the seeds in a bin
   if (ordered) {
-    KF_CUDA_TRY(ctx, launch_bin_points(ba, bins->n_events, s));
+    KF_CUDA_TRY(ctx, launch_bin_points(ba, ctx->num_sms, s));
     // perm holds ids within each event: make them global seed indices
     // (the seeds of event e start at seed_off[e])
     globalise_perm_kernel<<<int((S + 255) / 256), 256, 0, s>>>(perm, evt, seed_off, S);

@@ -196,7 +196,7 @@ struct EventLayout {
   // device offsets
   size_t d_par, d_cov, d_q, d_shits, d_sval, d_fpar, d_flo, d_fcov, d_fst, d_xyz, d_segoff, d_sseg, d_bhits, d_boff,
       d_bid, d_perm, d_candA, d_candB, d_hp, d_hh, d_rpar, d_rcov, d_rchi, d_rnh, d_rst, d_rhit, d_qpar, d_qcov,
-      d_qchi, d_qst, d_gxyz, d_gval, d_bcur, d_sboff, d_fine, d_total;
+      d_qchi, d_qst, d_gxyz, d_gval, d_sboff, d_fine, d_total;
   // host input / output block offsets
   size_t h_par, h_cov, h_q, h_shits, h_sval, h_xyz, h_segoff, h_in_total;
   size_t o_par, o_cov, o_chi, o_nh, o_st, o_hit, o_qpar, o_qcov, o_qchi, o_qst, h_out_total;
@@ -248,7 +248,6 @@ struct EventLayout {
     d_qst = take(refit ? n * 4 : 0);
     d_gxyz = take(refit ? L * 3 * n * 4 : 0);
     d_gval = take(refit ? L * n : 0);
-    d_bcur = take(size_t(Lb) * KF_NBINS * 4);     // binning cursors (hits, then seeds)
     d_sboff = take(size_t(KF_NBINS + 1) * 4);  // seed bin offsets
     d_fine = take(fine ? size_t(Lb) * (KF_NBINS_FINE + 1) * 4 : 0);  // hit sub-bin starts (register-resident build)
     d_total = o;
@@ -381,7 +380,7 @@ static cudaError_t prepare_batch(Serve* sv, const std::vector<Request*>& rs) {
   char* dslot = sv->d_table + kTableBytes * kRing + kPrepBytes * size_t(slot);
   FitEvent* hf = reinterpret_cast<FitEvent*>(hslot);
   BinSegment* hb = reinterpret_cast<BinSegment*>(hslot + kPrepFitBytes);
-  int64_t tracks = 0;
+  int64_t tracks = 0, points = 0;
   int segs = 0;
   for (size_t k = 0; k < rs.size(); ++k) {
     Request* r = rs[k];
@@ -422,6 +421,8 @@ static cudaError_t prepare_batch(Serve* sv, const std::vector<Request*>& rs) {
       b.stride = L.nh;
       b.p0 = hoff[l];
       b.p1 = std::min<int64_t>(hoff[l + 1], L.nh);
+      b.begin = points;
+      points += b.p1 - b.p0;
       b.bin_off = reinterpret_cast<int32_t*>(d + L.d_boff) + int64_t(l) * (KF_NBINS + 1);
       b.fine_off = L.fine ? reinterpret_cast<int32_t*>(d + L.d_fine) + int64_t(l) * (KF_NBINS_FINE + 1) : nullptr;
       b.out_pts = reinterpret_cast<float4*>(d + L.d_bhits);
@@ -447,7 +448,7 @@ static cudaError_t prepare_batch(Serve* sv, const std::vector<Request*>& rs) {
   fa.mass = ctx->mass;
   e = launch_fit_fused_table(fa, df, int(rs.size()), tracks, s);
   // the build's results do not depend on the order of the hits inside a bin
-  if (e == cudaSuccess) e = launch_bin_segment_table(db, segs, sub_bins, s);
+  if (e == cudaSuccess) e = launch_bin_segment_table(db, segs, points, sub_bins, s);
   if (e != cudaSuccess) return e;
   // (a register-resident build takes the seeds in their order, from the fit)
   for (size_t k = 0; k < rs.size() && sv->tune.build_scan != 4; ++k) {
@@ -464,9 +465,10 @@ static cudaError_t prepare_batch(Serve* sv, const std::vector<Request*>& rs) {
     sb.out_pts = nullptr;
     sb.out_id = reinterpret_cast<int32_t*>(d + L.d_perm);
     sb.out_seg = nullptr;
-    sb.cursor = reinterpret_cast<int32_t*>(d + L.d_bcur);
     sb.unordered = 1;  // the build's results do not depend on the order inside a bin
-    e = launch_bin_points(sb, 1, s);
+    sb.n_seg = 1;
+    sb.n_points = n;
+    e = launch_bin_points(sb, ctx->num_sms, s);
     if (e != cudaSuccess) return e;
     BuildInitArgs ia;
     ia.out = cand_at(d + L.d_candA, n);
