@@ -391,7 +391,7 @@ int kf_fit_f64(kf_ctx* ctx, const kf_tracks_f64* seeds, const kf_track_hits* hit
       a.v2 = sz * sz;
       a.first = l == 0;
       a.last = l == L - 1;
-      KF_CUDA_TRY(ctx, launch_fit_f64(a, s));
+      KF_CUDA_TRY(ctx, launch_fit_f64(a, ctx->num_sms, s));
     }
   }
   return KF_OK;

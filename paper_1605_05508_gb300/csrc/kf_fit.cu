@@ -36,6 +36,7 @@ constexpr int kFitWarpsPerSM = 24;
 constexpr int kFitTableBlocksPerSM = 5;
 constexpr int kNewtonF32 = 12;  // iteration cap of the safeguarded Newton solve
 constexpr int kNewtonF64 = 16;
+constexpr int kF64MinBlock = 32;
 
 // Positive-definiteness of the rank-5 covariance: Cholesky of P C P^T where P
 // maps to (t . pos, z, px, py, pz), t the transverse tangent of the cylinder
@@ -419,11 +420,16 @@ cudaError_t launch_fit_mixed(const FitFusedArgs& a, cudaStream_t st) {
   return cudaGetLastError();
 }
 
-cudaError_t launch_fit_f64(const FitF64Args& a, cudaStream_t st) {
+// Threads per block: as many as spread the event over all SMs, 32 to 128.  The
+// FP64 pipe serves under two lanes a cycle and SM, so an event's few warps side
+// by side on one SM wait for each other while other SMs idle.
+cudaError_t launch_fit_f64(const FitF64Args& a, int num_sms, cudaStream_t st) {
   const int64_t cnt = a.end - a.begin;
   if (cnt <= 0) return cudaSuccess;
-  const int grid = int((cnt + kFitThreads - 1) / kFitThreads);
-  fit_f64_kernel<<<grid, kFitThreads, 0, st>>>(a);
+  int block = kFitThreads;
+  while (block > kF64MinBlock && cnt < int64_t(num_sms) * block) block /= 2;
+  const int grid = int((cnt + block - 1) / block);
+  fit_f64_kernel<<<grid, block, 0, st>>>(a);
   return cudaGetLastError();
 }
 

@@ -194,7 +194,7 @@ struct FitEvent {
 // launch; a's arrays are ignored, its layers and constants used.
 cudaError_t launch_fit_fused_table(const FitFusedArgs& a, const FitEvent* table, int n_events, int64_t n_total,
                                    cudaStream_t st);
-cudaError_t launch_fit_f64(const FitF64Args& a, cudaStream_t st);
+cudaError_t launch_fit_f64(const FitF64Args& a, int num_sms, cudaStream_t st);
 
 // Hits of all layers per seed for a re-fit (kf_refit.cu): seeding layers from
 // the seed hits, building layers by the build's hit ids.
