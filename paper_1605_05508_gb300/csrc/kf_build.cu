@@ -1087,15 +1087,12 @@ __device__ __forceinline__ void merge_children(const uint32_t (&X)[W], const int
     return;
   }
   // entries of the warp's longest list (uniform)
-  const bool deep1 = __any_sync(kFull, X[1] != kNoChild);
   const bool deep2 = W > 2 && __any_sync(kFull, X[W > 2 ? 2 : 0] != kNoChild);
   const bool deep3 = W > 3 && __any_sync(kFull, X[W > 3 ? 3 : 0] != kNoChild);
   int rank[W];
 #pragma unroll
   for (int t = 0; t < W; ++t) rank[t] = t;
-  if (!deep1)
-    count_before<W, 1>(X, nhk, k, gbase, seg, rank);
-  else if (!deep2)
+  if (!deep2)
     count_before<W, 2>(X, nhk, k, gbase, seg, rank);
   else if (!deep3)
     count_before<W, (W < 3 ? W : 3)>(X, nhk, k, gbase, seg, rank);
@@ -1147,6 +1144,7 @@ template <int W, bool TABLE, bool MAT>
 __global__ void __launch_bounds__(kResThreads, resident_blocks_per_sm(W))
     build_resident_kernel(const __grid_constant__ BuildResidentArgs A) {
   constexpr int G = 32 / W;  // seeds per group
+  extern __shared__ int s_hist[];  // [n_layers][kResThreads]: hit id + 1 | parent rank << 24 (kHistLayers)
   __shared__ float4 s_stage[kScanStage * kResThreads];
   __shared__ int4 s_slots[W > 1 ? kResThreads : 1];
   int4* const slots = s_slots + (W > 1 ? int(threadIdx.x & ~31u) : 0);
@@ -1160,6 +1158,7 @@ __global__ void __launch_bounds__(kResThreads, resident_blocks_per_sm(W))
   // seeds (a few events), whose hits stay in L2, and a warp whose groups
   // happened to be cheap takes more (measured: 2 % faster at N = 6, 6 % at
   // N = 1 than a fixed grid stride)
+  const bool paths = A.paths != 0;
   auto next_group = [&]() {
     unsigned long long v = 0;
     if (lane == 0) v = atomicAdd(A.group_counter, 1ull);
@@ -1177,28 +1176,28 @@ __global__ void __launch_bounds__(kResThreads, resident_blocks_per_sm(W))
     const int64_t j = (TABLE ? gi - B.group_begin : n_groups - 1 - gi) * G + g;
     const bool seed_ok = g < G && j < B.S;
     int e = 0, nc = 0;
-    int64_t si = 0;  // seed index
     float a = A.a_scale;
     if (seed_ok) {
       e = B.seed_evt ? B.seed_evt[j] : 0;
-      si = B.seed_perm ? B.seed_perm[j] : j;
-      a = A.a_scale * float(B.charge[si]);
-      nc = B.seed_par ? 1 : B.in.ncand[j];
+      a = A.a_scale * float(B.charge[j]);
+      nc = W == 1 ? 1 : B.in.ncand[j];
     }
     bool active = seed_ok && k < nc;
+    // (lanes without a candidate load a valid one's state and never use it)
     float p[6], lo[3], C[21];
     float chi2tot = 0.f;
     int nh = 0;
     int32_t st = 0;
-    if (active && B.seed_par) {  // the seed itself
+    if constexpr (W == 1) {  // the seed itself
+      const int64_t i = active ? j : 0;
 #pragma unroll
-      for (int c = 0; c < 6; ++c) p[c] = B.seed_par[c * B.S + si];
+      for (int c = 0; c < 6; ++c) p[c] = B.seed_par[c * B.S + i];
 #pragma unroll
-      for (int c = 0; c < 3; ++c) lo[c] = B.seed_lo ? B.seed_lo[c * B.S + si] : 0.f;
+      for (int c = 0; c < 3; ++c) lo[c] = B.seed_lo ? B.seed_lo[c * B.S + i] : 0.f;
 #pragma unroll
-      for (int c = 0; c < 21; ++c) C[c] = B.seed_cov[c * B.S + si];
-    } else if (active) {
-      const int64_t slot = cand_slot(j, k, B.S, A.in_rm);
+      for (int c = 0; c < 21; ++c) C[c] = B.seed_cov[c * B.S + i];
+    } else {  // the first layer's children
+      const int64_t slot = active ? cand_slot(j, k, B.S, A.in_rm) : cand_slot(0, 0, B.S, A.in_rm);
 #pragma unroll
       for (int c = 0; c < 6; ++c) p[c] = B.in.par[c * S8 + slot];
 #pragma unroll
@@ -1209,13 +1208,7 @@ __global__ void __launch_bounds__(kResThreads, resident_blocks_per_sm(W))
       const int32_t meta = B.in.meta[slot];
       nh = meta & 0xff;
       st = meta >> 8;
-    } else {
-#pragma unroll
-      for (int c = 0; c < 6; ++c) p[c] = 0.f;
-#pragma unroll
-      for (int c = 0; c < 3; ++c) lo[c] = 0.f;
-#pragma unroll
-      for (int c = 0; c < 21; ++c) C[c] = 0.f;
+      if (paths) s_hist[threadIdx.x] = B.hist_hit[slot] + 1;  // of the first layer's launch
     }
     int n_win = nc;
     for (int l = A.l0; l < A.n_layers; ++l) {
@@ -1261,105 +1254,97 @@ __global__ void __launch_bounds__(kResThreads, resident_blocks_per_sm(W))
       merge_children<W>(X, P, nhk, A.max_cands, k, g * W, seg, slots, w, n_win);
       // materialise: lane k takes its winner's parent prediction and S^-1
       const int src = w.meta >= 0 ? g * W + (w.meta & 7) : lane;
-      float q[6], ql[3], qC[21], qS[6];
-      auto take = [&](auto v) {
-        if constexpr (W > 1)
-          return __shfl_sync(kFull, v, src);
-        else
-          return v;  // one lane a seed: its own prediction
-      };
+      if constexpr (W > 1) {
 #pragma unroll
-      for (int c = 0; c < 6; ++c) q[c] = take(p[c]);
+        for (int c = 0; c < 6; ++c) p[c] = __shfl_sync(kFull, p[c], src);
 #pragma unroll
-      for (int c = 0; c < 3; ++c) ql[c] = take(lo[c]);
+        for (int c = 0; c < 3; ++c) lo[c] = __shfl_sync(kFull, lo[c], src);
 #pragma unroll
-      for (int c = 0; c < 21; ++c) qC[c] = take(C[c]);
+        for (int c = 0; c < 21; ++c) C[c] = __shfl_sync(kFull, C[c], src);
 #pragma unroll
-      for (int c = 0; c < 6; ++c) qS[c] = take(Si[c]);
-      const int32_t pst = take(st);
-      const int pstopped = take(int(stopped));
+        for (int c = 0; c < 6; ++c) Si[c] = __shfl_sync(kFull, Si[c], src);
+        st = __shfl_sync(kFull, st, src);
+        stopped = __shfl_sync(kFull, int(stopped), src) != 0;
+      }
       active = seed_ok && w.meta >= 0;
       if (active) {
         int hit = -1;
-        int32_t st_new = pst;
         if (w.pos >= 0) {
           const float4 m = B.hits[h0 + w.pos];
           hit = __float_as_int(m.w);
           float r0, r1, r2;
-          kf::residual<float, true>(q, ql, m.x, m.y, m.z, r0, r1, r2);
-          kf::kalman_update<float, true>(q, ql, qC, qS, r0, r1, r2, A.v0, A.v1, A.v2);
-        } else if (!pstopped) {
-          st_new |= KF_ST_NO_HIT;
+          kf::residual<float, true>(p, lo, m.x, m.y, m.z, r0, r1, r2);
+          kf::kalman_update<float, true>(p, lo, C, Si, r0, r1, r2, A.v0, A.v1, A.v2);
+        } else if (!stopped) {
+          st |= KF_ST_NO_HIT;
         }
-        const int64_t hslot = int64_t(l) * S8 + cand_slot(j, k, B.S, l + 1 < A.rm_buffers);
-        B.hist_parent[hslot] = int8_t(w.meta & 7);
-        B.hist_hit[hslot] = hit;
-#pragma unroll
-        for (int c = 0; c < 6; ++c) p[c] = q[c];
-#pragma unroll
-        for (int c = 0; c < 3; ++c) lo[c] = ql[c];
-#pragma unroll
-        for (int c = 0; c < 21; ++c) C[c] = qC[c];
+        if (paths) {
+          s_hist[l * kResThreads + threadIdx.x] = (hit + 1) | (w.meta & 7) << 24;
+        } else {
+          const int64_t hslot = int64_t(l) * S8 + cand_slot(j, k, B.S, l + 1 < A.rm_buffers);
+          B.hist_parent[hslot] = int8_t(w.meta & 7);
+          B.hist_hit[hslot] = hit;
+        }
         chi2tot = __uint_as_float(w.x);
         nh = w.meta >> 8;
-        st = st_new;
       }
     }
-    if (B.res.best.par) {
-      // the final selection in place: lane k holds rank k, so the seed's
-      // first lane writes the best candidate and every lane below max_cands
-      // its summary; the paths (a chain of dependent history loads a seed)
-      // are left to build_final_kernel in its paths-only form, and with
-      // several lanes a seed so is the positive-definiteness check of the
-      // best covariance (its code here, run by one lane of W, cost 6 % of the
-      // N = 6 build): that kernel reads the position's low part from the
-      // candidate buffer
-      const kf_build_result& o = B.res;
-      if (seed_ok && k < A.max_cands) {
-        const int64_t seed = si;
-        const bool have = k < n_win;
-        if (k == 0) {
-#pragma unroll
-          for (int c = 0; c < 6; ++c) o.best.par[c * B.S + seed] = p[c];
-          if (o.best.par_lo)
-#pragma unroll
-            for (int c = 0; c < 3; ++c) o.best.par_lo[c * B.S + seed] = lo[c];
-#pragma unroll
-          for (int c = 0; c < 21; ++c) o.best.cov[c * B.S + seed] = C[c];
-          if (o.chi2_tot) o.chi2_tot[seed] = chi2tot;
-          if (o.n_hits) o.n_hits[seed] = nh;
-          if constexpr (W == 1) {
-            float pf[6];
-#pragma unroll
-            for (int c = 0; c < 3; ++c) pf[c] = p[c] + lo[c];
-#pragma unroll
-            for (int c = 3; c < 6; ++c) pf[c] = p[c];
-            if (o.status) o.status[seed] = pd5_final(pf, C) ? st : st | KF_ST_NOT_PD;
-          } else if (o.status) {
-            o.status[seed] = st;
-            const int64_t slot = cand_slot(j, 0, B.S, A.out_rm);
-#pragma unroll
-            for (int c = 0; c < 3; ++c) B.out.par[(6 + c) * S8 + slot] = lo[c];
-          }
-          if (o.n_cands) o.n_cands[seed] = n_win;
+    // the final selection in place: lane k holds rank k, so the seed's
+    // first lane writes the best candidate and its path, walked back through
+    // the history in shared memory (a pass of its own over a history in global
+    // memory, a chain of dependent loads a seed, took 11 us of one event's
+    // build), and every lane below max_cands its summary
+    // With several lanes a seed the positive-definiteness check of the best
+    // covariance is left to build_final_kernel (its code here, run by one lane
+    // of W, cost 6 % of the N = 6 build): that kernel reads the position's low
+    // part from the candidate buffer
+    const kf_build_result& o = B.res;
+    if (paths) {
+      __syncwarp();
+      if (seed_ok && k == 0 && o.hit_idx) {
+        const int* at = s_hist + (A.n_layers - 1) * kResThreads + threadIdx.x;  // lane 0 of the seed
+        int32_t* to = o.hit_idx + int64_t(A.n_layers - 1) * B.S + j;
+        int kk = 0;
+#pragma unroll 1
+        for (int l = A.n_layers - 1; l >= 0; --l, at -= kResThreads, to -= B.S) {
+          const int v = at[kk];
+          *to = (v & 0xffffff) - 1;
+          kk = v >> 24;
         }
-        const int64_t oc = seed * A.max_cands + k;
-        if (o.cand_chi2_tot) o.cand_chi2_tot[oc] = have ? chi2tot : 0.f;
-        if (o.cand_n_hits) o.cand_n_hits[oc] = have ? nh : 0;
       }
-    } else {
-      // the candidates after the last layer, for the final selection
-      if (active) {
-        const int64_t slot = cand_slot(j, k, B.S, A.out_rm);
+      __syncwarp();  // the history is read before the next group's
+    }
+    if (seed_ok && k < A.max_cands) {
+      const int64_t seed = j;
+      const bool have = k < n_win;
+      if (k == 0) {
 #pragma unroll
-        for (int c = 0; c < 6; ++c) B.out.par[c * S8 + slot] = p[c];
+        for (int c = 0; c < 6; ++c) o.best.par[c * B.S + seed] = p[c];
+        if (o.best.par_lo)
 #pragma unroll
-        for (int c = 0; c < 3; ++c) B.out.par[(6 + c) * S8 + slot] = lo[c];
+          for (int c = 0; c < 3; ++c) o.best.par_lo[c * B.S + seed] = lo[c];
 #pragma unroll
-        for (int c = 0; c < 21; ++c) B.out.cov[c * S8 + slot] = C[c];
-        B.out.chi2[slot] = chi2tot;
-        B.out.meta[slot] = nh | (st << 8);
+        for (int c = 0; c < 21; ++c) o.best.cov[c * B.S + seed] = C[c];
+        if (o.chi2_tot) o.chi2_tot[seed] = chi2tot;
+        if (o.n_hits) o.n_hits[seed] = nh;
+        if constexpr (W == 1) {
+          float pf[6];
+#pragma unroll
+          for (int c = 0; c < 3; ++c) pf[c] = p[c] + lo[c];
+#pragma unroll
+          for (int c = 3; c < 6; ++c) pf[c] = p[c];
+          if (o.status) o.status[seed] = pd5_final(pf, C) ? st : st | KF_ST_NOT_PD;
+        } else if (o.status) {
+          o.status[seed] = st;
+          const int64_t slot = cand_slot(j, 0, B.S, A.out_rm);
+#pragma unroll
+          for (int c = 0; c < 3; ++c) B.out.par[(6 + c) * S8 + slot] = lo[c];
+        }
+        if (o.n_cands) o.n_cands[seed] = n_win;
       }
+      const int64_t oc = seed * A.max_cands + k;
+      if (o.cand_chi2_tot) o.cand_chi2_tot[oc] = have ? chi2tot : 0.f;
+      if (o.cand_n_hits) o.cand_n_hits[oc] = have ? nh : 0;
     }
     if (seed_ok && k == 0) B.out.ncand[j] = int8_t(n_win);
   }
@@ -1388,37 +1373,32 @@ __global__ void __launch_bounds__(kResThreads, kResBlocksPerSM)
   if (j >= B.S) return;
   const int64_t S8 = B.S * kGroup;
   const int l = A.l0;
-  const int e = B.seed_evt ? B.seed_evt[j] : 0;
-  const int64_t si = B.seed_perm ? B.seed_perm[j] : j;
-  const float a = A.a_scale * float(B.charge[si]);
+  if (t == 0) *A.group_counter = 0;
+  const float a = A.a_scale * float(B.charge[j]);
   float p[6], lo[3], C[21];
-  float chi2tot = 0.f;
-  int nh = 0;
   int32_t st = 0;
-  if (B.seed_par) {  // the seed itself
 #pragma unroll
-    for (int c = 0; c < 6; ++c) p[c] = B.seed_par[c * B.S + si];
+  for (int c = 0; c < 6; ++c) p[c] = B.seed_par[c * B.S + j];
 #pragma unroll
-    for (int c = 0; c < 3; ++c) lo[c] = B.seed_lo ? B.seed_lo[c * B.S + si] : 0.f;
+  for (int c = 0; c < 3; ++c) lo[c] = B.seed_lo ? B.seed_lo[c * B.S + j] : 0.f;
 #pragma unroll
-    for (int c = 0; c < 21; ++c) C[c] = B.seed_cov[c * B.S + si];
-  } else {
-    const int64_t slot = cand_slot(j, 0, B.S, A.in_rm);  // the seed's only candidate
-#pragma unroll
-    for (int c = 0; c < 6; ++c) p[c] = B.in.par[c * S8 + slot];
-#pragma unroll
-    for (int c = 0; c < 3; ++c) lo[c] = B.in.par[(6 + c) * S8 + slot];
-#pragma unroll
-    for (int c = 0; c < 21; ++c) C[c] = B.in.cov[c * S8 + slot];
-    chi2tot = B.in.chi2[slot];
-    const int32_t meta = B.in.meta[slot];
-    nh = meta & 0xff;
-    st = meta >> 8;
+  for (int c = 0; c < 21; ++c) C[c] = B.seed_cov[c * B.S + j];
+  int e = 0;  // the seed's event
+  if (B.seed_off) {
+    int hi = B.n_events;
+    while (hi - e > 1) {
+      const int mid = (e + hi) >> 1;
+      if (B.seed_off[mid] <= j)
+        e = mid;
+      else
+        hi = mid;
+    }
+    B.evt_out[j] = e;
   }
   const int64_t sg = int64_t(e) * A.n_layers + l;
   const int64_t h0 = B.seg_off[sg];
-  bool stopped = (st & KF_ST_STOPPED) != 0;
-  if (!stopped) {
+  bool stopped = false;
+  {
     const int r = kf::propagate<float, kNewtonBuild, true, true>(p, lo, C, a, A.R[l]);
     if (r) {
       st |= r;
@@ -1440,14 +1420,14 @@ __global__ void __launch_bounds__(kResThreads, kResBlocksPerSM)
     const int32_t* boff = B.fine_off ? B.fine_off + sg * (KF_NBINS_FINE + 1) : B.bin_off + sg * (KF_NBINS + 1);
     int e0 = 0, e1 = -1, fa0 = 0, fa1 = nphi - 1, fb0 = 0, fb1 = -1;
     hit_window(p, lo, C, A.R[l], A.v0, A.v1, A.v2, A.cut, e0, e1, fa0, fa1, fb0, fb1, nphi);
-    scan_children(p, lo, C, A.v0, A.v1, A.v2, Si, e0, e1, fa0, fa1, fb0, fb1, boff, B.hits + h0, A.cut, chi2tot, X, P,
+    scan_children(p, lo, C, A.v0, A.v1, A.v2, Si, e0, e1, fa0, fa1, fb0, fb1, boff, B.hits + h0, A.cut, 0.f, X, P,
                   nphi, s_stage + threadIdx.x);
   }
   // no compatible hit (or a stopped seed): one child without a hit
-  int nhk = nh + 1;
+  int nhk = 1;
   if (X[0] == kNoChild) {
-    X[0] = __float_as_uint(chi2tot);
-    nhk = nh;
+    X[0] = __float_as_uint(0.f);
+    nhk = 0;
   }
   int n_win = 0;
 #pragma unroll 1
@@ -1489,7 +1469,7 @@ __global__ void __launch_bounds__(kResThreads, kResBlocksPerSM)
     for (int c = 0; c < 21; ++c) B.out.cov[c * S8 + os] = qC[c];
     B.out.chi2[os] = __uint_as_float(x);
     B.out.meta[os] = nhk | (st_new << 8);
-    B.hist_parent[int64_t(l) * S8 + os] = 0;
+    if (!A.paths) B.hist_parent[int64_t(l) * S8 + os] = 0;
     B.hist_hit[int64_t(l) * S8 + os] = hit;
   }
   B.out.ncand[j] = int8_t(n_win);
@@ -1511,12 +1491,13 @@ cudaError_t launch_build_first_layer(const BuildResidentArgs& a, cudaStream_t st
 
 template <bool TABLE, bool MAT>
 static void launch_resident_w(const BuildResidentArgs& a, int W, int grid, cudaStream_t st) {
+  const size_t hist = a.paths ? size_t(a.n_layers) * kResThreads * sizeof(int) : 0;
   switch (W) {
-    case 1: build_resident_kernel<1, TABLE, MAT><<<grid, kResThreads, 0, st>>>(a); break;
-    case 2: build_resident_kernel<2, TABLE, MAT><<<grid, kResThreads, 0, st>>>(a); break;
-    case 4: build_resident_kernel<4, TABLE, MAT><<<grid, kResThreads, 0, st>>>(a); break;
-    case 6: build_resident_kernel<6, TABLE, MAT><<<grid, kResThreads, 0, st>>>(a); break;
-    default: build_resident_kernel<8, TABLE, MAT><<<grid, kResThreads, 0, st>>>(a); break;
+    case 1: build_resident_kernel<1, TABLE, MAT><<<grid, kResThreads, hist, st>>>(a); break;
+    case 2: build_resident_kernel<2, TABLE, MAT><<<grid, kResThreads, hist, st>>>(a); break;
+    case 4: build_resident_kernel<4, TABLE, MAT><<<grid, kResThreads, hist, st>>>(a); break;
+    case 6: build_resident_kernel<6, TABLE, MAT><<<grid, kResThreads, hist, st>>>(a); break;
+    default: build_resident_kernel<8, TABLE, MAT><<<grid, kResThreads, hist, st>>>(a); break;
   }
 }
 
@@ -1556,8 +1537,8 @@ __global__ void build_final_kernel(const BuildFinalArgs A) {
   const bool last_rm = A.n_layers < A.rm_buffers;  // layout of buffer n_layers
   const int nc = A.cand.ncand[j];
   const kf_build_result& o = A.out;
-  if (A.paths_only) {  // the build launch wrote the rest but these
-    if (A.paths_only == 2 && o.status) {  // the best covariance positive definite (low part from the buffer)
+  if (A.rest) {  // build_resident_kernel wrote the others
+    if ((A.rest & 2) && o.status) {  // the best covariance positive definite (low part from the buffer)
       const int64_t slot = cand_slot(j, 0, A.S, last_rm);
       float pf[6], C[21];
       for (int c = 0; c < 6; ++c) pf[c] = o.best.par[c * A.S + seed];
@@ -1565,6 +1546,7 @@ __global__ void build_final_kernel(const BuildFinalArgs A) {
       for (int c = 0; c < 21; ++c) C[c] = o.best.cov[c * A.S + seed];
       if (!pd5_final(pf, C)) o.status[seed] |= KF_ST_NOT_PD;
     }
+    if (!(A.rest & 1)) return;
     if (o.hit_idx) {
       int kk = 0;
       for (int l = A.n_layers - 1; l >= 0; --l) {
@@ -1686,9 +1668,12 @@ cudaError_t launch_build_final(const BuildFinalArgs& a, cudaStream_t st) {
   return cudaGetLastError();
 }
 
-// evt[j] = the event of seed j: the last e with seed_off[e] <= j (binary search)
-__global__ void seed_event_kernel(int32_t* evt, const int64_t* seed_off, int64_t E, int64_t S) {
+// evt[j] = the event of seed j: the last e with seed_off[e] <= j (binary
+// search); and the group counter of the launch that follows set to zero
+__global__ void seed_event_kernel(int32_t* evt, const int64_t* seed_off, int64_t E, int64_t S,
+                                  unsigned long long* counter) {
   const int64_t j = int64_t(blockIdx.x) * blockDim.x + threadIdx.x;
+  if (j == 0) *counter = 0;
   if (j >= S) return;
   int64_t lo = 0, hi = E;
   while (hi - lo > 1) {
@@ -1757,10 +1742,6 @@ extern "C" int kf_build(kf_ctx* ctx, const kf_tracks* seeds, const int64_t* seed
   // of seeds spans a few events whose hits stay in L2 either way), and the
   // ordering launches are saved.
   const bool ordered = ctx->tune.build_scan != 4;
-  if (!ordered) {
-    seed_event_kernel<<<int((S + 255) / 256), 256, 0, s>>>(evt, seed_off, bins->n_events, S);
-    KF_CUDA_TRY(ctx, cudaGetLastError());
-  }
   BinArgs ba;
   ba.xyz = seeds->par;
   ba.stride = S;
@@ -1779,7 +1760,7 @@ extern "C" int kf_build(kf_ctx* ctx, const kf_tracks* seeds, const int64_t* seed
     globalise_perm_kernel<<<int((S + 255) / 256), 256, 0, s>>>(perm, evt, seed_off, S);
     KF_CUDA_TRY(ctx, cudaGetLastError());
   }
-  if (ctx->tune.build_scan != 4) {  // (the register-resident build reads the seeds itself)
+  if (ordered) {  // (the register-resident build reads the seeds itself)
     BuildInitArgs ia;
     ia.out = bufA;
     ia.par = seeds->par;
@@ -1796,9 +1777,93 @@ extern "C" int kf_build(kf_ctx* ctx, const kf_tracks* seeds, const int64_t* seed
   // candidate-packed steps: seeds spread over whole waves of blocks (build_pack_seeds)
   const int pack_seeds = build_pack_seeds(S, ctx->tune.build_scan, max_cands, ctx->num_sms);
   const int grid = pack_seeds > 0 ? int((S + pack_seeds - 1) / pack_seeds) : build_step_blocks(S, ctx->tune.build_scan);
+  const int rm_buffers = rank_major_buffers(max_cands, L);
+  if (ctx->tune.build_scan == 4) {
+    // register-resident layout: one launch takes every seed through all
+    // layers from the seeds themselves and selects the best candidates; with
+    // several lanes a seed, the first layer (one candidate a seed) runs first
+    // with one thread per seed, into buffer 1
+    BuildResidentArgs ra;
+    ra.one.in = bufA;
+    ra.one.out = bufB;
+    ra.one.hist_parent = hist_parent;
+    ra.one.hist_hit = hist_hit;
+    ra.one.seed_evt = evt;
+    ra.one.seed_off = seed_off;
+    ra.one.n_events = bins->n_events;
+    ra.one.evt_out = evt;
+    ra.one.charge = seeds->charge;
+    ra.one.hits = reinterpret_cast<const float4*>(bins->hits);
+    ra.one.bin_off = bins->bin_off;
+    ra.one.seg_off = bins->seg_off;
+    ra.one.fine_off = bins->fine_off;
+    ra.one.S = S;
+    ra.one.group_begin = 0;
+    ra.one.seed_begin = 0;
+    std::memset(&ra.one.res, 0, sizeof ra.one.res);
+    ra.one.seed_par = seeds->par;
+    ra.one.seed_lo = seeds->par_lo;
+    ra.one.seed_cov = seeds->cov;
+    ra.table = nullptr;
+    ra.n_batches = 1;
+    ra.n_groups = 0;
+    ra.n_seeds = 0;
+    ra.n_layers = L;
+    ra.l0 = 0;
+    ra.paths = resident_paths(L, out->cand_hit_idx != nullptr);
+    ra.rm_buffers = rm_buffers;
+    ra.max_cands = max_cands;
+    ra.in_rm = 0 < rm_buffers;
+    ra.out_rm = L < rm_buffers;
+    ra.a_scale = float(kCLight * double(ctx->cfg.bz_tesla));
+    ra.v0 = v0;
+    ra.v1 = v0;
+    ra.v2 = v2;
+    ra.cut = ctx->cfg.chi2_cut;
+    ra.mass = ctx->mass;
+    for (int l = 0; l < kMaxLayers; ++l) {
+      ra.R[l] = l < L ? ctx->radius[bins->first_layer + l] : 0.f;
+      ra.x_x0[l] = l < L ? ctx->x_x0[bins->first_layer + l] : 0.f;
+    }
+    ra.group_counter = reinterpret_cast<unsigned long long*>(base + total - b_ctr);
+    if (resident_lanes(max_cands) > 1) {
+      // the first layer with one thread per seed (buffer 0 -> buffer 1), then
+      // layers 1 .. L-1 from buffer 1 into the other buffer
+      BuildResidentArgs fl = ra;
+      fl.out_rm = 1 < rm_buffers;
+      KF_CUDA_TRY(ctx, launch_build_first_layer(fl, s));
+      ra.one.seed_par = ra.one.seed_lo = ra.one.seed_cov = nullptr;
+      ra.one.in = bufB;
+      ra.in_rm = 1 < rm_buffers;
+      ra.one.out = bufA;
+      ra.l0 = 1;
+    } else {
+      seed_event_kernel<<<int((S + 255) / 256), 256, 0, s>>>(evt, seed_off, bins->n_events, S, ra.group_counter);
+      KF_CUDA_TRY(ctx, cudaGetLastError());
+    }
+    // the last launch also selects the best candidates and writes `out`, all
+    // but what resident_rest() names
+    ra.one.res = *out;
+    KF_CUDA_TRY(ctx, launch_build_resident(ra, ctx->num_sms, s));
+    BuildFinalArgs fa;
+    fa.cand = ra.one.out;
+    fa.hist_parent = hist_parent;
+    fa.hist_hit = hist_hit;
+    fa.seed_perm = nullptr;
+    fa.S = S;
+    fa.n_layers = L;
+    fa.max_cands = max_cands;
+    fa.rm_buffers = rm_buffers;
+    fa.rest = resident_rest(max_cands, L, out->cand_hit_idx != nullptr);
+    fa.out = *out;
+    if (((fa.rest & 1) && (out->hit_idx || out->cand_hit_idx)) || ((fa.rest & 2) && out->status)) {
+      build_final_kernel<<<int((S + 127) / 128), 128, 0, s>>>(fa);
+      KF_CUDA_TRY(ctx, cudaGetLastError());
+    }
+    return KF_OK;
+  }
   // one slot (the whole batch) per layer launch; the table goes to device
   // scratch in one copy (the host array is consumed before the call returns)
-  const int rm_buffers = rank_major_buffers(max_cands, L);
   std::vector<BuildSlot> table(L);
   for (int l = 0; l < L; ++l) {
     BuildSlot& d = table[l];
@@ -1830,86 +1895,6 @@ extern "C" int kf_build(kf_ctx* ctx, const kf_tracks* seeds, const int64_t* seed
   // next buffer could overwrite what a block still on the previous layer
   // reads in the same memory.  Layers up to the switch run one launch each.
   // The grouped layouts launch once per layer.
-  if (ctx->tune.build_scan == 4) {
-    // register-resident layout: one launch takes every seed through all
-    // layers from the seeds themselves and selects the best candidates; with
-    // several lanes a seed, the first layer (one candidate a seed) runs first
-    // with one thread per seed, into buffer 1
-    BuildResidentArgs ra;
-    ra.one.in = bufA;
-    ra.one.out = bufB;
-    ra.one.hist_parent = hist_parent;
-    ra.one.hist_hit = hist_hit;
-    ra.one.seed_evt = evt;
-    ra.one.seed_perm = nullptr;  // the given order
-    ra.one.charge = seeds->charge;
-    ra.one.hits = reinterpret_cast<const float4*>(bins->hits);
-    ra.one.bin_off = bins->bin_off;
-    ra.one.seg_off = bins->seg_off;
-    ra.one.fine_off = bins->fine_off;
-    ra.one.S = S;
-    ra.one.group_begin = 0;
-    ra.one.seed_begin = 0;
-    std::memset(&ra.one.res, 0, sizeof ra.one.res);
-    ra.one.seed_par = seeds->par;
-    ra.one.seed_lo = seeds->par_lo;
-    ra.one.seed_cov = seeds->cov;
-    ra.table = nullptr;
-    ra.n_batches = 1;
-    ra.n_groups = 0;
-    ra.n_seeds = 0;
-    ra.n_layers = L;
-    ra.l0 = 0;
-    ra.rm_buffers = rm_buffers;
-    ra.max_cands = max_cands;
-    ra.in_rm = 0 < rm_buffers;
-    ra.out_rm = L < rm_buffers;
-    ra.a_scale = float(kCLight * double(ctx->cfg.bz_tesla));
-    ra.v0 = v0;
-    ra.v1 = v0;
-    ra.v2 = v2;
-    ra.cut = ctx->cfg.chi2_cut;
-    ra.mass = ctx->mass;
-    for (int l = 0; l < kMaxLayers; ++l) {
-      ra.R[l] = l < L ? ctx->radius[bins->first_layer + l] : 0.f;
-      ra.x_x0[l] = l < L ? ctx->x_x0[bins->first_layer + l] : 0.f;
-    }
-    if (resident_lanes(max_cands) > 1 && L > 1) {
-      // the first layer with one thread per seed (buffer 0 -> buffer 1), then
-      // layers 1 .. L-1 from buffer 1 into the other buffer
-      BuildResidentArgs fl = ra;
-      fl.out_rm = 1 < rm_buffers;
-      KF_CUDA_TRY(ctx, launch_build_first_layer(fl, s));
-      ra.one.seed_par = ra.one.seed_lo = ra.one.seed_cov = nullptr;
-      ra.one.in = bufB;
-      ra.in_rm = 1 < rm_buffers;
-      ra.one.out = bufA;
-      ra.l0 = 1;
-    }
-    // the last launch also selects the best candidates and writes `out`,
-    // all but the paths and the covariance check: those follow, one thread
-    // a seed
-    ra.one.res = *out;
-    ra.group_counter = reinterpret_cast<unsigned long long*>(base + total - b_ctr);
-    KF_CUDA_TRY(ctx, cudaMemsetAsync(ra.group_counter, 0, sizeof(unsigned long long), s));
-    KF_CUDA_TRY(ctx, launch_build_resident(ra, ctx->num_sms, s));
-    BuildFinalArgs fa;
-    fa.cand = ra.one.out;
-    fa.hist_parent = hist_parent;
-    fa.hist_hit = hist_hit;
-    fa.seed_perm = nullptr;
-    fa.S = S;
-    fa.n_layers = L;
-    fa.max_cands = max_cands;
-    fa.rm_buffers = rm_buffers;
-    fa.paths_only = resident_defers_pd(max_cands) ? 2 : 1;
-    fa.out = *out;
-    if (out->hit_idx || out->cand_hit_idx || (out->status && fa.paths_only == 2)) {
-      build_final_kernel<<<int((S + 127) / 128), 128, 0, s>>>(fa);
-      KF_CUDA_TRY(ctx, cudaGetLastError());
-    }
-    return KF_OK;
-  }
   const int first_fused = is_packed(ctx->tune.build_scan) ? (rm_buffers > L ? 0 : std::min(L, rm_buffers)) : L;
   for (int l = 0; l < (first_fused < L ? first_fused + 1 : L); ++l) {
     const bool fused = l == first_fused;
@@ -1939,7 +1924,7 @@ extern "C" int kf_build(kf_ctx* ctx, const kf_tracks* seeds, const int64_t* seed
   fa.n_layers = L;
   fa.max_cands = max_cands;
   fa.rm_buffers = rm_buffers;
-  fa.paths_only = 0;
+  fa.rest = 0;
   fa.out = *out;
   build_final_kernel<<<int((S + 127) / 128), 128, 0, s>>>(fa);
   KF_CUDA_TRY(ctx, cudaGetLastError());

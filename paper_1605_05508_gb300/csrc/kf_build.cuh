@@ -98,8 +98,9 @@ struct BuildFinalArgs {
   int64_t S;
   int n_layers, max_cands;
   int rm_buffers;  // rank_major_buffers(max_cands, n_layers)
-  int paths_only;  // 1: only the paths (hit_idx, cand_hit_idx; of cand only ncand is read),
-                   // 2: also the best covariance check (status; cand: ncand, rank 0's low part)
+  int rest;  // after build_resident_kernel, what it left (0: the whole selection): bit 0, the paths
+             // (hit_idx, cand_hit_idx; of cand only ncand is read); bit 1, the best covariance
+             // check (status; of cand rank 0's low part)
   kf_build_result out;
 };
 
@@ -166,9 +167,13 @@ struct ResidentBatch {
   CandBuf out;               // buffer n_layers (layout out_rm); must not alias `in`
   int8_t* hist_parent;       // [n_layers][S8]: layer l's slots in the layout of buffer l + 1
   int32_t* hist_hit;         // [n_layers][S8]
-  const int32_t* seed_evt;   // [S] sorted position -> event, or null (event 0)
-  const int32_t* seed_perm;  // [S] sorted position -> seed index, or null (the identity)
-  const int8_t* charge;      // [S] by seed index
+  const int32_t* seed_evt;   // [S] seed -> event, or null (event 0)
+  // first-layer launch, when set: the seeds' events by searching seed_off
+  // ([n_events + 1]), written to evt_out ([S])
+  const int64_t* seed_off;
+  int32_t n_events;
+  int32_t* evt_out;
+  const int8_t* charge;      // [S]
   const float4* hits;
   const int32_t* bin_off;
   const int64_t* seg_off;
@@ -178,16 +183,16 @@ struct ResidentBatch {
   int64_t S;
   int64_t group_begin;       // with a table: the launch's first group of this batch
   int64_t seed_begin;        // with a table: the first-layer launch's first seed of this batch
-  // the seeds themselves ([6] / [3] (or null: zero) / [21] x S, by seed
-  // index), read in place of buffer `in` when set (then l0 = 0: every seed
-  // one candidate, chi2 0, no hit)
+  // the seeds themselves ([6] / [3] (or null: zero) / [21] x S): read by the
+  // first-layer launch, and with one lane a seed by build_resident_kernel (l0
+  // = 0), which else reads the first layer's children from `in` (l0 = 1)
   const float* seed_par;
   const float* seed_lo;
   const float* seed_cov;
-  // the final selection, done by the kernel after the last layer when
-  // res.best.par is set (the best candidate and the optional per-candidate
-  // summaries, as build_final_kernel writes them, all but the paths; only
-  // out.ncand is then written); else the candidates go to `out`
+  // the final selection, done by the kernel after the last layer: the best
+  // candidate and the optional per-candidate summaries, as build_final_kernel
+  // writes them, all but what resident_rest() leaves (of `out` only ncand and
+  // rank 0's low part are written)
   kf_build_result res;
 };
 struct BuildResidentArgs {
@@ -198,11 +203,12 @@ struct BuildResidentArgs {
   int64_t n_seeds;                   // with a table: seeds of all its batches
   int n_layers, l0, rm_buffers, max_cands;
   int in_rm, out_rm;
+  int paths;  // 1: the history in shared memory and the best paths written (resident_paths)
   float a_scale, v0, v1, v2, cut, mass;
   float R[kMaxLayers];     // building layer radii
   float x_x0[kMaxLayers];  // building layer thickness in radiation lengths (0: none)
   // device counter, zero at launch: the warps fetch their next seed group
-  // from it (build_resident_kernel)
+  // from it (build_resident_kernel); the first-layer launch sets it to zero
   unsigned long long* group_counter;
 };
 // Lanes per seed of the resident layout for max_cands (1, 2, 4, 6 or 8).
@@ -212,6 +218,15 @@ inline int resident_lanes(int max_cands) {
 // With several lanes a seed, the resident layout leaves the best covariance's
 // positive-definiteness check to the final kernel (paths_only = 2).
 inline bool resident_defers_pd(int max_cands) { return resident_lanes(max_cands) > 1; }
+// The history of a group's candidates stays in shared memory for up to this
+// many building layers, and build_resident_kernel then writes the best paths
+// itself; when every candidate's path is wanted it goes to global memory.
+constexpr int kHistLayers = 16;
+inline bool resident_paths(int n_layers, bool cand_paths) { return n_layers <= kHistLayers && !cand_paths; }
+// What build_resident_kernel leaves to build_final_kernel (BuildFinalArgs::rest).
+inline int resident_rest(int max_cands, int n_layers, bool cand_paths) {
+  return (resident_paths(n_layers, cand_paths) ? 0 : 1) | (resident_defers_pd(max_cands) ? 2 : 0);
+}
 // seeds per warp group of the resident layout (32 / lanes per seed)
 inline int resident_group(int max_cands) { return 32 / resident_lanes(max_cands); }
 cudaError_t launch_build_resident(const BuildResidentArgs& a, int num_sms, cudaStream_t st);

@@ -307,7 +307,7 @@ constexpr size_t kCounterBytes = 256;
 // layer (one candidate a seed) with one thread per seed, seeds -> buffer B,
 // and the rest from buffer B into buffer A; else one launch, seeds -> B.
 inline bool resident_split(const kf_serve_config& c) {
-  return resident_lanes(c.max_cands) > 1 && c.n_build_layers > 1;
+  return resident_lanes(c.max_cands) > 1;
 }
 
 struct Serve {
@@ -531,9 +531,11 @@ static ResidentBatch resident_batch_of(Serve* sv, Request* r, bool first) {
   b.hist_parent = reinterpret_cast<int8_t*>(d + L.d_hp);
   b.hist_hit = reinterpret_cast<int32_t*>(d + L.d_hh);
   b.seed_evt = nullptr;
+  b.seed_off = nullptr;  // one event
+  b.n_events = 1;
+  b.evt_out = nullptr;
   // seeds in their given order (one event's hits stay in L2 whatever the
   // order), read straight from the seed fit's output
-  b.seed_perm = nullptr;
   b.charge = reinterpret_cast<const int8_t*>(d + L.d_q);
   b.hits = reinterpret_cast<const float4*>(d + L.d_bhits);
   b.bin_off = reinterpret_cast<const int32_t*>(d + L.d_boff);
@@ -585,7 +587,7 @@ static cudaError_t finish(Serve* sv, Request* r) {
   fa.n_layers = L.Lb;
   fa.max_cands = sv->cfg.max_cands;
   fa.rm_buffers = rank_major_buffers(sv->cfg.max_cands, L.Lb);
-  fa.paths_only = resident ? (resident_defers_pd(sv->cfg.max_cands) ? 2 : 1) : 0;
+  fa.rest = resident ? resident_rest(sv->cfg.max_cands, L.Lb, false) : 0;
   fa.out.best.n = n;
   fa.out.best.par = reinterpret_cast<float*>(d + L.d_rpar);
   fa.out.best.par_lo = nullptr;
@@ -594,7 +596,7 @@ static cudaError_t finish(Serve* sv, Request* r) {
   fa.out.n_hits = reinterpret_cast<int32_t*>(d + L.d_rnh);
   fa.out.status = reinterpret_cast<int32_t*>(d + L.d_rst);
   fa.out.hit_idx = reinterpret_cast<int32_t*>(d + L.d_rhit);
-  cudaError_t e = launch_build_final(fa, s);
+  cudaError_t e = resident && fa.rest == 0 ? cudaSuccess : launch_build_final(fa, s);
   if (e == cudaSuccess && L.refit) {
     // re-fit: every seed's hits over all layers, then one fused fit launch
     // from the vertex seed (the same arithmetic as kf_refit / kf_fit)
@@ -794,6 +796,7 @@ static void scheduler(Serve* sv) {
       ra.n_batches = int(nb);
       const int Lb = sv->cfg.n_build_layers, Ls = sv->cfg.n_seed_layers;
       ra.n_layers = Lb;
+      ra.paths = resident_paths(Lb, false);
       ra.max_cands = sv->cfg.max_cands;
       ra.rm_buffers = rank_major_buffers(ra.max_cands, Lb);
       ra.a_scale = float(kCLight * double(sv->ctx->cfg.bz_tesla));
@@ -805,6 +808,10 @@ static void scheduler(Serve* sv) {
         ra.R[l] = sv->ctx->radius[Ls + l];
         ra.x_x0[l] = sv->ctx->x_x0[Ls + l];
       }
+      ra.group_counter = reinterpret_cast<unsigned long long*>(sv->d_table + kTableBytes * kRing +
+                                                               kPrepBytes * kPrepRing + kCounterBytes * ring);
+      if (e == cudaSuccess && !split)  // (else the first-layer launch sets it)
+        e = cudaMemsetAsync(ra.group_counter, 0, sizeof(unsigned long long), sv->stream);
       if (e == cudaSuccess && split) {
         BuildResidentArgs fl = ra;
         fl.table = df;
@@ -816,9 +823,6 @@ static void scheduler(Serve* sv) {
       }
       ra.table = dt;
       ra.n_groups = groups;
-      ra.group_counter = reinterpret_cast<unsigned long long*>(sv->d_table + kTableBytes * kRing +
-                                                               kPrepBytes * kPrepRing + kCounterBytes * ring);
-      if (e == cudaSuccess) e = cudaMemsetAsync(ra.group_counter, 0, sizeof(unsigned long long), sv->stream);
       ra.l0 = split ? 1 : 0;
       ra.in_rm = ra.l0 < ra.rm_buffers;
       ra.out_rm = Lb < ra.rm_buffers;
