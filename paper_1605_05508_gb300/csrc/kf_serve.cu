@@ -93,10 +93,12 @@ class Arena {
   size_t size_ = 0, used_ = 0, peak_ = 0;
 };
 
-// Host threads that share the large copies of kf_submit: staging an event in
-// pinned memory is a few MB, and one thread copies at ~15 GB/s, far below
-// what the host memory delivers; the submitting thread takes chunks too and
-// returns when all of its event's chunks are done.
+// Host threads that share the large copies of kf_submit and kf_poll: an event
+// is a few MB in and out, and one thread copies at ~15 GB/s, far below what the
+// host memory delivers (13 GB/s into freshly allocated results, whose pages it
+// touches first); the calling thread takes chunks too and returns when all of
+// its event's chunks are done.  A small event is copied by the caller alone:
+// waking the others takes longer.
 class CopyPool {
  public:
   struct Piece {
@@ -117,6 +119,12 @@ class CopyPool {
     threads_.clear();
   }
   void copy(const Piece* pieces, int n_pieces) {
+    size_t total = 0;
+    for (int p = 0; p < n_pieces; ++p) total += pieces[p].bytes;
+    if (total <= kAlone) {
+      for (int p = 0; p < n_pieces; ++p) std::memcpy(pieces[p].dst, pieces[p].src, pieces[p].bytes);
+      return;
+    }
     Job job;
     std::vector<Chunk> chunks;
     for (int p = 0; p < n_pieces; ++p)
@@ -149,7 +157,7 @@ class CopyPool {
   }
 
  private:
-  static constexpr size_t kChunk = size_t(1) << 20;
+  static constexpr size_t kChunk = size_t(1) << 19, kAlone = size_t(1) << 18;
   struct Job {
     std::mutex m;
     std::condition_variable cv;
@@ -346,7 +354,8 @@ struct Serve {
   std::unordered_map<uint64_t, std::unique_ptr<Request>> all;
   kf_serve_stats stats{};
   kf_tuning tune{};  // launch parameters in effect at kf_serve_start
-  CopyPool copier;   // kf_submit's staging copies
+  CopyPool copier;   // kf_submit's staging copies and kf_poll's result copies
+  int polling = 0;   // result copies under way, outside the lock
 };
 
 static void fail_all_locked(Serve* sv, int err) {
@@ -920,6 +929,10 @@ void kf_serve_shutdown_internal(kf_ctx* ctx) {
   }
   sv->cv.notify_all();
   if (sv->thread.joinable()) sv->thread.join();
+  {
+    std::unique_lock<std::mutex> lk(sv->mu);
+    sv->done_cv.wait(lk, [&] { return sv->polling == 0; });
+  }
   sv->copier.stop();
   cudaSetDevice(ctx->device);
   if (sv->stream) cudaStreamSynchronize(sv->stream);
@@ -1100,8 +1113,12 @@ int kf_poll(kf_ctx* ctx, uint64_t ticket, kf_event_result* out, int64_t timeout_
   std::unique_lock<std::mutex> lk(sv->mu);
   auto it = sv->all.find(ticket);
   if (it == sv->all.end()) return KF_EINVAL;
-  Request* r = it->second.get();
-  auto ready = [&] { return r->state == kDone || r->state == kFailed; };
+  // looked up anew at every wake-up: a submission may rehash the table, and
+  // another poller may take the ticket
+  auto ready = [&] {
+    it = sv->all.find(ticket);
+    return it == sv->all.end() || it->second->state == kDone || it->second->state == kFailed;
+  };
   if (!ready()) {
     if (timeout_us == 0) return KF_ETIMEDOUT;
     if (timeout_us < 0)
@@ -1109,6 +1126,8 @@ int kf_poll(kf_ctx* ctx, uint64_t ticket, kf_event_result* out, int64_t timeout_
     else if (!sv->done_cv.wait_for(lk, std::chrono::microseconds(timeout_us), ready))
       return KF_ETIMEDOUT;
   }
+  if (it == sv->all.end()) return KF_EINVAL;
+  Request* r = it->second.get();
   if (r->state == kFailed) {
     release_locked(sv, r);
     if (r->has_out) sv->harena.release(r->h_out_off, r->lay.h_out_total);
@@ -1118,30 +1137,41 @@ int kf_poll(kf_ctx* ctx, uint64_t ticket, kf_event_result* out, int64_t timeout_
     sv->all.erase(it);
     return KF_ECUDA;
   }
+  // the ticket is taken; its results are copied outside the lock, so that the
+  // scheduler and the submitters go on meanwhile
+  const std::unique_ptr<Request> taken = std::move(it->second);
+  sv->all.erase(it);
+  sv->polling++;
+  lk.unlock();
   const EventLayout& L = r->lay;
   const char* o = sv->hmem + r->h_out_off;
-  const int64_t n = L.n;
-  if (out->best_par) std::memcpy(out->best_par, o + L.o_par, 6 * n * 4);
-  if (out->best_cov) std::memcpy(out->best_cov, o + L.o_cov, 21 * n * 4);
-  if (out->chi2_tot) std::memcpy(out->chi2_tot, o + L.o_chi, n * 4);
-  if (out->n_hits) std::memcpy(out->n_hits, o + L.o_nh, n * 4);
-  if (out->status) std::memcpy(out->status, o + L.o_st, n * 4);
-  if (out->hit_idx) std::memcpy(out->hit_idx, o + L.o_hit, size_t(L.Lb) * n * 4);
+  const size_t n = size_t(L.n), Lall = size_t(L.ns + L.Lb);
+  CopyPool::Piece pieces[10];
+  int np = 0;
+  auto piece = [&](void* dst, size_t at, size_t bytes) {
+    if (dst) pieces[np++] = {dst, o + at, bytes};
+  };
+  piece(out->best_par, L.o_par, 6 * n * 4);
+  piece(out->best_cov, L.o_cov, 21 * n * 4);
+  piece(out->chi2_tot, L.o_chi, n * 4);
+  piece(out->n_hits, L.o_nh, n * 4);
+  piece(out->status, L.o_st, n * 4);
+  piece(out->hit_idx, L.o_hit, size_t(L.Lb) * n * 4);
   if (L.refit) {
-    const size_t Lall = size_t(L.ns + L.Lb);
-    if (out->refit_par) std::memcpy(out->refit_par, o + L.o_qpar, 6 * n * 4);
-    if (out->refit_cov) std::memcpy(out->refit_cov, o + L.o_qcov, 21 * n * 4);
-    if (out->refit_chi2) std::memcpy(out->refit_chi2, o + L.o_qchi, Lall * n * 4);
-    if (out->refit_status) std::memcpy(out->refit_status, o + L.o_qst, n * 4);
+    piece(out->refit_par, L.o_qpar, 6 * n * 4);
+    piece(out->refit_cov, L.o_qcov, 21 * n * 4);
+    piece(out->refit_chi2, L.o_qchi, Lall * n * 4);
+    piece(out->refit_status, L.o_qst, n * 4);
   }
+  sv->copier.copy(pieces, np);
   out->latency_ms = std::chrono::duration<double, std::milli>(r->t_done - r->t_submit).count();
   out->queued_ms = std::chrono::duration<double, std::milli>(r->t_admit - r->t_submit).count();
-  release_locked(sv, r);
-  sv->harena.release(r->h_out_off, L.h_out_total);
-  r->has_out = false;
   if (r->done) cudaEventDestroy(r->done);
   if (r->prepped) cudaEventDestroy(r->prepped);
-  sv->all.erase(it);
+  lk.lock();
+  release_locked(sv, r);
+  sv->harena.release(r->h_out_off, L.h_out_total);
+  if (--sv->polling == 0) sv->done_cv.notify_all();
   return KF_OK;
 }
 
