@@ -8,6 +8,7 @@
 //   fit_fused_kernel        all layers in one launch, the track held in
 //                           registers (kf_fit, kf_fit_fused, kf_fit_noalloc;
 //                           fit_mixed_kernel: the mixed-precision form);
+//   fit_gather_kernel       the same over the hits a build chose (kf_refit);
 //   fit_layer_stage_kernel  one layer step over the whole batch (kf_fit with
 //                           kf_tuning.fit_stage replays one launch per layer
 //                           from a captured CUDA graph), each warp's next 32
@@ -32,7 +33,7 @@ constexpr int kFitThreads = 128;
 // layers' arithmetic is bound by instruction issue and register reads, not by
 // memory: 1.444 ms for 4M tracks x 10 layers against 1.472 at 20 warps.
 constexpr int kFitWarpsPerSM = 24;
-// with the table of events the index arithmetic takes the registers over 80
+// with the table of events, or gathered hits, the registers go over 80
 constexpr int kFitTableBlocksPerSM = 5;
 constexpr int kNewtonF32 = 12;  // iteration cap of the safeguarded Newton solve
 constexpr int kNewtonF64 = 16;
@@ -254,10 +255,90 @@ __global__ void __launch_bounds__(kStageThreads, kStageBlocksPerSM)
   }
 }
 
+// The hits of one track, layer after layer: get(l, ..) is called for l = 0, 1,
+// .. in turn and returns whether layer l has a hit.
+// From the fit's own arrays [L][3][n], valid [L][n] or null.
+struct ArrayHits {
+  const float* xyz;
+  const uint8_t* valid;
+  int64_t n, i;
+  __device__ __forceinline__ bool get(int l, float& m0, float& m1, float& m2) {
+    const float* h = xyz + int64_t(l) * 3 * n;
+    m0 = h[i];
+    m1 = h[n + i];
+    m2 = h[2 * n + i];
+    return valid ? valid[int64_t(l) * n + i] != 0 : true;
+  }
+};
+
+// Of a built track (kf_refit): the seeding layers from the seed's own hits,
+// the building layers by the ids the build chose, looked up in the raw hits of
+// the seed's event.  The lookups are two dependent loads, so the hit of the
+// next layer is fetched, and the id of the one after it, before a layer's
+// arithmetic.
+struct GatherHits {
+  const RefitGatherArgs& G;
+  int64_t i;
+  int e;
+  int32_t id;             // of the layer after the next
+  float nx, ny, nz;       // the next layer's hit
+  bool nok;
+
+  __device__ __forceinline__ GatherHits(const RefitGatherArgs& g, int64_t track) : G(g), i(track) {
+    int lo = 0, hi = G.E - 1;  // the event: seed_off[e] <= i < seed_off[e + 1]
+    while (lo < hi) {
+      const int mid = (lo + hi + 1) >> 1;
+      if (G.seed_off[mid] <= i)
+        lo = mid;
+      else
+        hi = mid - 1;
+    }
+    e = lo;
+    id = id_of(0);
+    fetch(0);
+  }
+  __device__ __forceinline__ int32_t id_of(int l) const {
+    const int b = l - G.Ls;
+    return b >= 0 && b < G.Lb ? G.hit_idx[int64_t(b) * G.n + i] : -1;
+  }
+  // the hit of layer l (its id in `id`) into nx .. nok, and the id of layer l + 1
+  __device__ __forceinline__ void fetch(int l) {
+    const int64_t n = G.n;
+    nx = ny = nz = 0.f;
+    nok = false;
+    if (l < G.Ls) {
+      const float* s = G.seed_xyz + int64_t(l) * 3 * n;
+      nx = s[i];
+      ny = s[n + i];
+      nz = s[2 * n + i];
+      nok = G.seed_valid ? G.seed_valid[int64_t(l) * n + i] != 0 : true;
+    } else if (id >= 0) {
+      const int64_t* seg = G.seg_off + int64_t(e) * G.Lb + (l - G.Ls);
+      const int64_t h = seg[0] + id;
+      if (h < seg[1] && h >= 0 && h < G.n_hits) {
+        nx = G.hit_xyz[h];
+        ny = G.hit_xyz[G.n_hits + h];
+        nz = G.hit_xyz[2 * G.n_hits + h];
+        nok = true;
+      }
+    }
+    id = id_of(l + 1);
+  }
+  __device__ __forceinline__ bool get(int l, float& m0, float& m1, float& m2) {
+    m0 = nx;
+    m1 = ny;
+    m2 = nz;
+    const bool ok = nok;
+    if (l + 1 < G.Ls + G.Lb) fetch(l + 1);
+    return ok;
+  }
+};
+
 // All layers of track i of the arrays of E (FitFusedArgs itself, or one
-// event of a table: the same field names), with the layers and constants of A.
-template <bool UPD64, class EV>
-__device__ __forceinline__ void fused_track(const EV& E, const FitFusedArgs& A, int64_t i) {
+// event of a table: the same field names), with the layers and constants of A
+// and the hits of H.
+template <bool UPD64, class EV, class HITS>
+__device__ __forceinline__ void fused_track(const EV& E, const FitFusedArgs& A, int64_t i, HITS H) {
   const int64_t n = E.n;
   {
     float p[6], lo[3], C[21];
@@ -272,10 +353,10 @@ __device__ __forceinline__ void fused_track(const EV& E, const FitFusedArgs& A, 
     for (int l = 0; l < A.n_layers; ++l) {
       float chi2 = -1.f;
       if (!(st & KF_ST_STOPPED)) {
-        const float* h = E.hits + int64_t(l) * 3 * n;
-        const bool has_hit = E.valid ? E.valid[int64_t(l) * n + i] != 0 : true;
-        st |= track_step<float, kNewtonF32, true, UPD64>(p, lo, C, a, A.R[l], A.x_x0[l], A.mass, has_hit, h[i],
-                                                         h[n + i], h[2 * n + i], A.v0, A.v1, A.v2, chi2);
+        float m0, m1, m2;
+        const bool has_hit = H.get(l, m0, m1, m2);
+        st |= track_step<float, kNewtonF32, true, UPD64>(p, lo, C, a, A.R[l], A.x_x0[l], A.mass, has_hit, m0, m1, m2,
+                                                         A.v0, A.v1, A.v2, chi2);
       }
       if (E.chi2) E.chi2[int64_t(l) * n + i] = chi2;
     }
@@ -295,13 +376,22 @@ __device__ __forceinline__ void fused_track(const EV& E, const FitFusedArgs& A, 
 template <int THREADS>
 __global__ void __launch_bounds__(THREADS, kFitWarpsPerSM * 32 / THREADS) fit_fused_kernel(const FitFusedArgs A) {
   const int64_t i = int64_t(blockIdx.x) * THREADS + threadIdx.x;
-  if (i < A.n) fused_track<false>(A, A, i);
+  if (i < A.n) fused_track<false>(A, A, i, ArrayHits{A.hits, A.valid, A.n, i});
 }
 
 // The mixed-precision form (kf_fit_mixed).
 __global__ void __launch_bounds__(kFitThreads, 1) fit_mixed_kernel(const FitFusedArgs A) {
   const int64_t i = int64_t(blockIdx.x) * kFitThreads + threadIdx.x;
-  if (i < A.n) fused_track<true>(A, A, i);
+  if (i < A.n) fused_track<true>(A, A, i, ArrayHits{A.hits, A.valid, A.n, i});
+}
+
+// The re-fit of built tracks: the fused fit over gathered hits (A's hit arrays
+// are not used).  A pass that gathers them into arrays first took 18 us of the
+// 79 us re-fit of 128 000 tracks over 10 layers.
+__global__ void __launch_bounds__(kFitThreads, kFitTableBlocksPerSM)
+    fit_gather_kernel(const FitFusedArgs A, const RefitGatherArgs G) {
+  const int64_t i = int64_t(blockIdx.x) * kFitThreads + threadIdx.x;
+  if (i < A.n) fused_track<false>(A, A, i, GatherHits(G, i));
 }
 
 // The fused fit of several events in one launch (the events a serving
@@ -313,7 +403,9 @@ __global__ void __launch_bounds__(kFitThreads, kFitTableBlocksPerSM)
   for (int64_t t = int64_t(blockIdx.x) * blockDim.x + threadIdx.x; t < n_total; t += stride) {
     int q = 0;
     while (q + 1 < n_events && table[q + 1].begin <= t) ++q;
-    fused_track<false>(table[q], A, t - table[q].begin);
+    const FitEvent& E = table[q];
+    const int64_t i = t - E.begin;
+    fused_track<false>(E, A, i, ArrayHits{E.hits, E.valid, E.n, i});
   }
 }
 
@@ -411,6 +503,12 @@ cudaError_t launch_fit_fused(const FitFusedArgs& a, int block, cudaStream_t st) 
     fit_fused_kernel<64><<<grid, 64, 0, st>>>(a);
   else
     fit_fused_kernel<128><<<grid, 128, 0, st>>>(a);
+  return cudaGetLastError();
+}
+
+cudaError_t launch_fit_gather(const FitFusedArgs& a, const RefitGatherArgs& g, cudaStream_t st) {
+  if (a.n <= 0) return cudaSuccess;
+  fit_gather_kernel<<<int((a.n + kFitThreads - 1) / kFitThreads), kFitThreads, 0, st>>>(a, g);
   return cudaGetLastError();
 }
 

@@ -53,7 +53,7 @@ struct kf_ctx {
   cudaStream_t capture_stream = nullptr;
   // scratch pools
   kfi::Scratch s_status, s_lo, s_host_in, s_host_out;
-  kfi::Scratch s_bin_id, s_build, s_refit, s_build64;
+  kfi::Scratch s_bin_id, s_build, s_build64;
   // graph cache
   std::vector<kfi::GraphEntry> graphs;
   uint64_t use_clock = 0;
@@ -196,8 +196,8 @@ cudaError_t launch_fit_fused_table(const FitFusedArgs& a, const FitEvent* table,
                                    cudaStream_t st);
 cudaError_t launch_fit_f64(const FitF64Args& a, int num_sms, cudaStream_t st);
 
-// Hits of all layers per seed for a re-fit (kf_refit.cu): seeding layers from
-// the seed hits, building layers by the build's hit ids.
+// Hits of all layers per seed for a re-fit: seeding layers from the seed hits,
+// building layers by the build's hit ids.
 struct RefitGatherArgs {
   const float* seed_xyz;      // [Ls][3][n]
   const uint8_t* seed_valid;  // [Ls][n] or null (all valid)
@@ -205,11 +205,9 @@ struct RefitGatherArgs {
   const float* hit_xyz;       // [3][n_hits]
   const int64_t* seg_off;     // [E * Lb + 1]
   const int32_t* hit_idx;     // [Lb][n]
-  float* xyz;                 // [Ls + Lb][3][n]
-  uint8_t* valid;             // [Ls + Lb][n]
   int64_t n, n_hits;
   int Ls, Lb, E;
 };
-cudaError_t launch_refit_gather(const RefitGatherArgs& a, cudaStream_t st);
+cudaError_t launch_fit_gather(const FitFusedArgs& a, const RefitGatherArgs& g, cudaStream_t st);
 
 }  // namespace kfi

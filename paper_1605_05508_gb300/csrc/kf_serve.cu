@@ -204,7 +204,7 @@ struct EventLayout {
   // device offsets
   size_t d_par, d_cov, d_q, d_shits, d_sval, d_fpar, d_flo, d_fcov, d_fst, d_xyz, d_segoff, d_sseg, d_bhits, d_boff,
       d_bid, d_perm, d_candA, d_candB, d_hp, d_hh, d_rpar, d_rcov, d_rchi, d_rnh, d_rst, d_rhit, d_qpar, d_qcov,
-      d_qchi, d_qst, d_gxyz, d_gval, d_sboff, d_fine, d_total;
+      d_qchi, d_qst, d_sboff, d_fine, d_total;
   // host input / output block offsets
   size_t h_par, h_cov, h_q, h_shits, h_sval, h_xyz, h_segoff, h_in_total;
   size_t o_par, o_cov, o_chi, o_nh, o_st, o_hit, o_qpar, o_qcov, o_qchi, o_qst, h_out_total;
@@ -254,8 +254,6 @@ struct EventLayout {
     d_qcov = take(refit ? 21 * n * 4 : 0);
     d_qchi = take(refit ? L * n * 4 : 0);
     d_qst = take(refit ? n * 4 : 0);
-    d_gxyz = take(refit ? L * 3 * n * 4 : 0);
-    d_gval = take(refit ? L * n : 0);
     d_sboff = take(size_t(KF_NBINS + 1) * 4);  // seed bin offsets
     d_fine = take(fine ? size_t(Lb) * (KF_NBINS_FINE + 1) * 4 : 0);  // hit sub-bin starts (register-resident build)
     d_total = o;
@@ -607,8 +605,7 @@ static cudaError_t finish(Serve* sv, Request* r) {
   fa.out.hit_idx = reinterpret_cast<int32_t*>(d + L.d_rhit);
   cudaError_t e = resident && fa.rest == 0 ? cudaSuccess : launch_build_final(fa, s);
   if (e == cudaSuccess && L.refit) {
-    // re-fit: every seed's hits over all layers, then one fused fit launch
-    // from the vertex seed (the same arithmetic as kf_refit / kf_fit)
+    // re-fit from the vertex seed over all layers, as kf_refit
     RefitGatherArgs g;
     g.seed_xyz = reinterpret_cast<const float*>(d + L.d_shits);
     g.seed_valid = reinterpret_cast<const uint8_t*>(d + L.d_sval);
@@ -616,41 +613,23 @@ static cudaError_t finish(Serve* sv, Request* r) {
     g.hit_xyz = reinterpret_cast<const float*>(d + L.d_xyz);
     g.seg_off = reinterpret_cast<const int64_t*>(d + L.d_segoff);
     g.hit_idx = reinterpret_cast<const int32_t*>(d + L.d_rhit);
-    g.xyz = reinterpret_cast<float*>(d + L.d_gxyz);
-    g.valid = reinterpret_cast<uint8_t*>(d + L.d_gval);
     g.n = n;
     g.n_hits = L.nh;
     g.Ls = L.ns;
     g.Lb = L.Lb;
     g.E = 1;
-    e = launch_refit_gather(g, s);
-    if (e == cudaSuccess) {
-      kf_ctx* ctx = sv->ctx;
-      FitFusedArgs q;
-      std::memset(&q, 0, sizeof q);
-      q.in_par = reinterpret_cast<const float*>(d + L.d_par);
-      q.in_lo = nullptr;
-      q.in_cov = reinterpret_cast<const float*>(d + L.d_cov);
-      q.charge = reinterpret_cast<const int8_t*>(d + L.d_q);
-      q.out_par = reinterpret_cast<float*>(d + L.d_qpar);
-      q.out_lo = nullptr;
-      q.out_cov = reinterpret_cast<float*>(d + L.d_qcov);
-      q.hits = g.xyz;
-      q.valid = g.valid;
-      q.chi2 = reinterpret_cast<float*>(d + L.d_qchi);
-      q.status = reinterpret_cast<int32_t*>(d + L.d_qst);
-      q.n = n;
-      q.n_layers = L.ns + L.Lb;
-      q.a_scale = float(kCLight * double(ctx->cfg.bz_tesla));
-      q.v0 = q.v1 = ctx->cfg.sigma_xy_cm * ctx->cfg.sigma_xy_cm;
-      q.v2 = ctx->cfg.sigma_z_cm * ctx->cfg.sigma_z_cm;
-      for (int l = 0; l < L.ns + L.Lb; ++l) {
-        q.R[l] = ctx->radius[l];
-        q.x_x0[l] = ctx->x_x0[l];
-      }
-      q.mass = ctx->mass;
-      e = launch_fit_fused(q, sv->tune.fit_block, s);
-    }
+    kf_tracks seeds = {}, fitted = {};
+    seeds.n = n;
+    seeds.par = reinterpret_cast<float*>(d + L.d_par);
+    seeds.cov = reinterpret_cast<float*>(d + L.d_cov);
+    seeds.charge = reinterpret_cast<int8_t*>(d + L.d_q);
+    fitted.par = reinterpret_cast<float*>(d + L.d_qpar);
+    fitted.cov = reinterpret_cast<float*>(d + L.d_qcov);
+    kf_track_hits all = {};
+    all.n_layers = L.ns + L.Lb;
+    e = launch_fit_gather(fused_args(sv->ctx, &seeds, &all, &fitted, reinterpret_cast<float*>(d + L.d_qchi),
+                                     reinterpret_cast<int32_t*>(d + L.d_qst)),
+                          g, s);
   }
   // results are contiguous on the device (rpar .. rhit, then the re-fit's)
   // and in the output block
