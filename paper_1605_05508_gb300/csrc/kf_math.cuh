@@ -86,6 +86,36 @@ KF_HD float div_fast(float a, float b) {
 }
 KF_HD double div_fast(double a, double b) { return a / b; }
 
+// ---- pairs: two single-precision operations in one instruction on sm_103a,
+// each rounded as by itself (so the bits are those of two scalar ones).  A
+// three-register fused multiply-add is bound by the reads of its operands (46
+// TFLOP/s measured against 74 with two of them constant); on pairs of registers
+// it reaches 58, and takes half the instructions.  The update and the first
+// half of the transport on pairs of rows take 4M tracks x 10 layers from 1 444
+// to 1 349 us and the build of 50 events from 1 133 to 1 061 us (with 14 fewer
+// registers); the second half (T1 J^T) would copy as many operands as it saves
+// instructions.
+struct F2 {
+  float x, y;
+};
+KF_HD F2 both(float a) { return {a, a}; }
+KF_HD F2 fma2(F2 a, F2 b, F2 c) {
+#ifdef __CUDA_ARCH__
+  const float2 r = __ffma2_rn(make_float2(a.x, a.y), make_float2(b.x, b.y), make_float2(c.x, c.y));
+  return {r.x, r.y};
+#else
+  return {fmaf(a.x, b.x, c.x), fmaf(a.y, b.y, c.y)};
+#endif
+}
+KF_HD F2 mul2(F2 a, F2 b) {
+#ifdef __CUDA_ARCH__
+  const float2 r = __fmul2_rn(make_float2(a.x, a.y), make_float2(b.x, b.y));
+  return {r.x, r.y};
+#else
+  return {a.x * b.x, a.y * b.y};
+#endif
+}
+
 // ---- masks and status words (one lane: bool and int32)
 template <typename T>
 struct Lanes {
@@ -323,6 +353,68 @@ KF_HD typename Lanes<T>::I propagate_lanes(T p[6], T lo[3], T C[21], T a, T R, t
   ok = ok & !tang;
   if (!any(ok)) return st;
 
+  // C' = J C J^T with T1 = J C (rows 0..4; row 5 of J is e_pz, and J[i][2] =
+  // (i == 2))
+  T J[5][6], T1[5][6];
+  if constexpr (!Lanes<T>::kDouble) {
+    // ---- surface Jacobian and T1 = J C as below, rows (0, 1) and (3, 4) in
+    // pairs, every element by the same operations in the same order
+    const float ip2 = ip * ip;
+    const float sp3 = (s * ip2) * ip;
+    const float thp2 = hp.th * ip2;
+    const F2 n01 = {-(hp.PX * sp3), -(hp.PY * sp3)}, n34 = {-(hp.PY * thp2), hp.PX * thp2};
+    const float n2 = -(pz * sp3);
+    const F2 bx = both(px), by = both(py), bz = both(pz);
+    const F2 D01[3] = {fma2(n01, bx, {hp.sa, -hp.ca}), fma2(n01, by, {hp.ca, hp.sa}), mul2(n01, bz)};
+    const F2 D34[3] = {fma2(n34, bx, {hp.cth, -hp.sth}), fma2(n34, by, {hp.sth, hp.cth}), mul2(n34, bz)};
+    const float D2[3] = {n2 * px, n2 * py, fmaf(n2, pz, s * ip)};
+    const float irp = rcp_t(rdotp);
+    const float iden = pmag * irp;
+    const float w0 = X * iden, w1 = Y * iden;
+    const F2 f01 = {-(hp.PX * ip), -(hp.PY * ip)}, f34 = {-(k * hp.PY), k * hp.PX};
+    const float f2 = -(pz * ip);
+    F2 J01[5], J34[5];  // columns 0, 1, 3, 4, 5
+    float J2[5];
+    J01[0] = {(Y * hp.PY) * irp, f01.y * w0};
+    J01[1] = {f01.x * w1, (X * hp.PX) * irp};
+    J34[0] = mul2(f34, both(w0));
+    J34[1] = mul2(f34, both(w1));
+    J2[0] = f2 * w0;
+    J2[1] = f2 * w1;
+#pragma unroll
+    for (int kk = 0; kk < 3; ++kk) {
+      const float w = fmaf(X, D01[kk].x, Y * D01[kk].y) * iden;
+      J01[2 + kk] = fma2(f01, both(w), D01[kk]);
+      J34[2 + kk] = fma2(f34, both(w), D34[kk]);
+      J2[2 + kk] = fmaf(f2, w, D2[kk]);
+    }
+#pragma unroll
+    for (int l = 0; l < 5; ++l) {
+      const int lc = l < 2 ? l : l + 1;
+      J[0][lc] = J01[l].x;
+      J[1][lc] = J01[l].y;
+      J[2][lc] = J2[l];
+      J[3][lc] = J34[l].x;
+      J[4][lc] = J34[l].y;
+    }
+#pragma unroll
+    for (int col = 0; col < 6; ++col) {
+      F2 a01 = mul2(J01[0], both(C[sym(0, col)])), a34 = mul2(J34[0], both(C[sym(0, col)]));
+      float a2 = fmaf(J2[0], C[sym(0, col)], C[sym(2, col)]);
+#pragma unroll
+      for (int l = 1; l < 5; ++l) {
+        const float c = C[sym(l < 2 ? l : l + 1, col)];
+        a01 = fma2(J01[l], both(c), a01);
+        a34 = fma2(J34[l], both(c), a34);
+        a2 = fmaf(J2[l], c, a2);
+      }
+      T1[0][col] = a01.x;
+      T1[1][col] = a01.y;
+      T1[2][col] = a2;
+      T1[3][col] = a34.x;
+      T1[4][col] = a34.y;
+    }
+  } else {
   // ---- surface Jacobian
   // fixed-s partials D (rows x, y, z, px, py over columns px0, py0, pz0)
   const T ip2 = ip * ip;
@@ -355,7 +447,6 @@ KF_HD typename Lanes<T>::I propagate_lanes(T p[6], T lo[3], T C[21], T a, T R, t
   // J[i][l] for i < 5 over columns l in {0,1,3,4,5}; J[i][2] = (i == 2).
   // The transverse 2x2 corner is written in its cancellation-free form
   // (1 - PX X / r.p = Y PY / r.p, ...).
-  T J[5][6];
 #pragma unroll
   for (int i = 0; i < 5; ++i) {
     J[i][0] = nf[i] * w[0];
@@ -367,8 +458,7 @@ KF_HD typename Lanes<T>::I propagate_lanes(T p[6], T lo[3], T C[21], T a, T R, t
   J[0][0] = (Y * hp.PY) * irp;
   J[1][1] = (X * hp.PX) * irp;
 
-  // ---- C' = J C J^T.  T1 = J C (rows 0..4); row 5 of J is e_pz.
-  T T1[5][6];
+  // T1 = J C
 #pragma unroll
   for (int i = 0; i < 5; ++i) {
 #pragma unroll
@@ -383,6 +473,7 @@ KF_HD typename Lanes<T>::I propagate_lanes(T p[6], T lo[3], T C[21], T a, T R, t
         }
       T1[i][col] = acc;
     }
+  }
   }
   T Cn[21];
 #pragma unroll
@@ -566,9 +657,102 @@ KF_HD void kalman_update_lanes(T p[6], T lo[3], T C[21], const T Si[6], T r0, T 
     }
 }
 
+// The same in single precision on pairs of rows (2r, 2r + 1), every element by
+// the same operations in the same order.
+template <bool EXT>
+KF_HD void kalman_update_pairs(float p[6], float lo[3], float C[21], const float Si[6], float r0, float r1, float r2,
+                               float v0, float v1, float v2) {
+  // columns 0, 1, 2 of C
+  const F2 c0[3] = {{C[0], C[1]}, {C[3], C[6]}, {C[10], C[15]}};
+  const F2 c1[3] = {{C[1], C[2]}, {C[4], C[7]}, {C[11], C[16]}};
+  const F2 c2[3] = {{C[3], C[4]}, {C[5], C[8]}, {C[12], C[17]}};
+  const F2 s0 = both(-Si[0]), s1 = both(-Si[1]), s2 = both(-Si[2]), s3 = both(-Si[3]), s4 = both(-Si[4]),
+           s5 = both(-Si[5]);
+  F2 k0[3], k1[3], k2[3];  // the negated gain's columns
+#pragma unroll
+  for (int r = 0; r < 3; ++r) {
+    k0[r] = fma2(c0[r], s0, fma2(c1[r], s1, mul2(c2[r], s3)));
+    k1[r] = fma2(c0[r], s1, fma2(c1[r], s2, mul2(c2[r], s4)));
+    k2[r] = fma2(c0[r], s3, fma2(c1[r], s4, mul2(c2[r], s5)));
+  }
+  float ndx[6];
+#pragma unroll
+  for (int r = 0; r < 3; ++r) {
+    const F2 d = fma2(k0[r], both(r0), fma2(k1[r], both(r1), mul2(k2[r], both(r2))));
+    ndx[2 * r] = d.x;
+    ndx[2 * r + 1] = d.y;
+  }
+#pragma unroll
+  for (int i = 0; i < 6; ++i) {
+    if (EXT && i < 3) {
+      float h, e;
+      two_sum(p[i], lo[i] - ndx[i], h, e);
+      p[i] = h;
+      lo[i] = e;
+    } else {
+      p[i] = p[i] - ndx[i];
+    }
+  }
+  // B = (I - K H) C': columns 0 .. 2 in full, of the others the rows from the
+  // diagonal on
+  auto b = [&](int r, F2 cij, float c0j, float c1j, float c2j) {
+    return fma2(k0[r], both(c0j), fma2(k1[r], both(c1j), fma2(k2[r], both(c2j), cij)));
+  };
+  F2 b0[3], b1[3], b2[3];
+#pragma unroll
+  for (int r = 0; r < 3; ++r) {
+    b0[r] = b(r, c0[r], C[0], C[1], C[3]);
+    b1[r] = b(r, c1[r], C[1], C[2], C[4]);
+    b2[r] = b(r, c2[r], C[3], C[4], C[5]);
+  }
+  const F2 b3 = b(2, {C[13], C[18]}, C[6], C[7], C[8]);
+  const F2 b4 = b(2, {C[14], C[19]}, C[10], C[11], C[12]);
+  const float b33 = fmaf(k0[1].y, C[6], fmaf(k1[1].y, C[7], fmaf(k2[1].y, C[8], C[9])));
+  const float b55 = fmaf(k0[2].y, C[15], fmaf(k1[2].y, C[16], fmaf(k2[2].y, C[17], C[20])));
+  F2 w0[3], w1[3], w2[3];  // nK V
+#pragma unroll
+  for (int r = 0; r < 3; ++r) {
+    w0[r] = mul2(k0[r], both(v0));
+    w1[r] = mul2(k1[r], both(v1));
+    w2[r] = mul2(k2[r], both(v2));
+  }
+  // element (i, j) = B_ij + (nK V)_i . nK_j + B_i . nK_j over columns 0 .. 2
+  auto c = [&](int r, F2 bij, float j0, float j1, float j2) {
+    F2 a = fma2(w0[r], both(j0), bij);
+    a = fma2(w1[r], both(j1), a);
+    a = fma2(w2[r], both(j2), a);
+    a = fma2(b0[r], both(j0), a);
+    a = fma2(b1[r], both(j1), a);
+    return fma2(b2[r], both(j2), a);
+  };
+  auto c1y = [&](int r, float bij, float j0, float j1, float j2) {  // row 2r + 1 alone
+    float a = fmaf(w0[r].y, j0, bij);
+    a = fmaf(w1[r].y, j1, a);
+    a = fmaf(w2[r].y, j2, a);
+    a = fmaf(b0[r].y, j0, a);
+    a = fmaf(b1[r].y, j1, a);
+    return fmaf(b2[r].y, j2, a);
+  };
+  const F2 n00 = c(0, b0[0], k0[0].x, k1[0].x, k2[0].x), n20 = c(1, b0[1], k0[0].x, k1[0].x, k2[0].x),
+           n40 = c(2, b0[2], k0[0].x, k1[0].x, k2[0].x);
+  const float n11 = c1y(0, b1[0].y, k0[0].y, k1[0].y, k2[0].y);
+  const F2 n21 = c(1, b1[1], k0[0].y, k1[0].y, k2[0].y), n41 = c(2, b1[2], k0[0].y, k1[0].y, k2[0].y);
+  const F2 n22 = c(1, b2[1], k0[1].x, k1[1].x, k2[1].x), n42 = c(2, b2[2], k0[1].x, k1[1].x, k2[1].x);
+  const float n33 = c1y(1, b33, k0[1].y, k1[1].y, k2[1].y);
+  const F2 n43 = c(2, b3, k0[1].y, k1[1].y, k2[1].y);
+  const F2 n44 = c(2, b4, k0[2].x, k1[2].x, k2[2].x);
+  const float n55 = c1y(2, b55, k0[2].y, k1[2].y, k2[2].y);
+  C[0] = n00.x, C[1] = n00.y, C[2] = n11, C[3] = n20.x, C[4] = n21.x, C[5] = n22.x, C[6] = n20.y, C[7] = n21.y;
+  C[8] = n22.y, C[9] = n33, C[10] = n40.x, C[11] = n41.x, C[12] = n42.x, C[13] = n43.x, C[14] = n44.x;
+  C[15] = n40.y, C[16] = n41.y, C[17] = n42.y, C[18] = n43.y, C[19] = n44.y, C[20] = n55;
+}
+
 template <typename T, bool EXT>
 KF_HD void kalman_update(T p[6], T lo[3], T C[21], const T Si[6], T r0, T r1, T r2, T v0, T v1, T v2) {
-  kalman_update_lanes<T, EXT>(p, lo, C, Si, r0, r1, r2, v0, v1, v2, true);
+  if constexpr (!Lanes<T>::kDouble)
+    kalman_update_pairs<EXT>(p, lo, C, Si, r0, r1, r2, v0, v1, v2);
+  else
+    kalman_update_lanes<T, EXT>(p, lo, C, Si, r0, r1, r2, v0, v1, v2, true);
 }
 
 // Mixed precision: the same update with S^-1, the gain and the Joseph
