@@ -657,6 +657,16 @@ __device__ __forceinline__ void child_insert(uint32_t (&X)[LW], int (&P)[LW], ui
     P[0] = u;
     return;
   }
+  if constexpr (LW > 1) {
+    if (X[1] == kNoChild && x != X[0]) {
+      const bool first = x < X[0];
+      X[1] = first ? X[0] : x;
+      P[1] = first ? P[0] : u;
+      X[0] = first ? x : X[0];
+      P[0] = first ? u : P[0];
+      return;
+    }
+  }
   bool lt[LW];  // the new child goes before entry t
   bool tie = false;
 #pragma unroll
