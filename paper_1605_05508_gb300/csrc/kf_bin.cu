@@ -164,6 +164,7 @@ __device__ __forceinline__ void bin_one_segment(const float* xyz, int64_t stride
 
 template <bool FINE>
 __global__ void __launch_bounds__(kScanThreads) bin_segment_kernel(const BinArgs A) {
+  chain_begin();
   extern __shared__ int cnt[];  // counts, then cursors (padded layout)
   __shared__ int warp_tot[32];
   const int seg = blockIdx.x;
@@ -224,12 +225,15 @@ __device__ __forceinline__ int segment_of(const BinArgs& A, int64_t g) {
 
 template <bool FINE>
 __global__ void __launch_bounds__(kPointThreads) bin_zero_kernel(const BinArgs A) {
-  const BinSegment S = segment<FINE>(A, int(blockIdx.y));
-  (FINE ? S.fine_off : S.bin_off)[blockIdx.x * kPointThreads + threadIdx.x] = 0;
+  chain_begin();
+  constexpr int kBlocks = (FINE ? KF_NBINS_FINE : KF_NBINS) / kPointThreads;
+  const BinSegment S = segment<FINE>(A, int(blockIdx.x) / kBlocks);
+  (FINE ? S.fine_off : S.bin_off)[int(blockIdx.x) % kBlocks * kPointThreads + threadIdx.x] = 0;
 }
 
 template <bool FINE>
 __global__ void __launch_bounds__(kPointThreads) bin_count_kernel(const BinArgs A) {
+  chain_begin();
   const int64_t g = int64_t(blockIdx.x) * kPointThreads + threadIdx.x;
   if (g >= A.n_points) return;
   const BinSegment S = segment<FINE>(A, segment_of(A, g));
@@ -243,6 +247,7 @@ __global__ void __launch_bounds__(kPointThreads) bin_count_kernel(const BinArgs 
 
 template <bool FINE>
 __global__ void __launch_bounds__(kScanThreads) bin_scan_kernel(const BinArgs A) {
+  chain_begin();
   constexpr int NB = FINE ? KF_NBINS_FINE : KF_NBINS;
   constexpr int kPer = NB / kScanThreads;
   extern __shared__ int cnt[];  // counts, then starts (padded layout)
@@ -282,6 +287,7 @@ __global__ void __launch_bounds__(kScanThreads) bin_scan_kernel(const BinArgs A)
 
 template <bool FINE>
 __global__ void __launch_bounds__(kPointThreads) bin_place_kernel(const BinArgs A) {
+  chain_begin();
   const int64_t g = int64_t(blockIdx.x) * kPointThreads + threadIdx.x;
   if (g >= A.n_points) return;
   const BinSegment S = segment<FINE>(A, segment_of(A, g));
@@ -303,6 +309,7 @@ __global__ void __launch_bounds__(kPointThreads) bin_place_kernel(const BinArgs 
 constexpr int kOrderRun = 128;
 constexpr int kOrderWarps = 4;
 __global__ void __launch_bounds__(32 * kOrderWarps) bin_order_kernel(const BinArgs A) {
+  chain_begin();
   __shared__ int s_id[kOrderWarps][kOrderRun];
   __shared__ int s_off[kOrderWarps][33];
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
@@ -391,17 +398,13 @@ static cudaError_t launch_bin_wide(const BinArgs& a, cudaStream_t st) {
   constexpr int smem = FINE ? kFineSmem : kScanSmem;
   cudaError_t e = segment_smem_attrs(bin_scan_kernel<FINE>, smem, attr_set);
   if (e != cudaSuccess) return e;
-  if (a.table)
-    bin_zero_kernel<FINE><<<dim3((FINE ? KF_NBINS_FINE : KF_NBINS) / kPointThreads, a.n_seg), kPointThreads, 0, st>>>(a);
-  else
-    e = cudaMemsetAsync(FINE ? a.fine_off : a.bin_off, 0,
-                        size_t(a.n_seg) * ((FINE ? KF_NBINS_FINE : KF_NBINS) + 1) * sizeof(int32_t), st);
-  if (e != cudaSuccess) return e;
+  const unsigned zero = unsigned(a.n_seg) * ((FINE ? KF_NBINS_FINE : KF_NBINS) / kPointThreads);
   const unsigned grid = unsigned((a.n_points + kPointThreads - 1) / kPointThreads);
-  if (grid > 0) bin_count_kernel<FINE><<<grid, kPointThreads, 0, st>>>(a);
-  bin_scan_kernel<FINE><<<a.n_seg, kScanThreads, smem, st>>>(a);
-  if (grid > 0) bin_place_kernel<FINE><<<grid, kPointThreads, 0, st>>>(a);
-  return cudaGetLastError();
+  e = launch_chained(bin_zero_kernel<FINE>, zero, kPointThreads, 0, st, a);
+  if (e == cudaSuccess && grid > 0) e = launch_chained(bin_count_kernel<FINE>, grid, kPointThreads, 0, st, a);
+  if (e == cudaSuccess) e = launch_chained(bin_scan_kernel<FINE>, a.n_seg, kScanThreads, smem, st, a);
+  if (e == cudaSuccess && grid > 0) e = launch_chained(bin_place_kernel<FINE>, grid, kPointThreads, 0, st, a);
+  return e;
 }
 
 cudaError_t launch_bin_segment_table(const BinSegment* table, int n, int64_t n_points, bool fine, cudaStream_t st) {
@@ -435,15 +438,15 @@ cudaError_t launch_bin_points(const BinArgs& a, int num_sms, cudaStream_t st) {
     static std::atomic<bool> seg_attr_set[kMaxDevices], fine_attr_set[kMaxDevices];
     if (a.fine_off) {
       e = segment_smem_attrs(bin_segment_kernel<true>, kFineSmem, fine_attr_set);
-      if (e == cudaSuccess) bin_segment_kernel<true><<<a.n_seg, kScanThreads, kFineSmem, st>>>(a);
+      if (e == cudaSuccess) e = launch_chained(bin_segment_kernel<true>, a.n_seg, kScanThreads, kFineSmem, st, a);
     } else {
       e = segment_smem_attrs(bin_segment_kernel<false>, kScanSmem, seg_attr_set);
-      if (e == cudaSuccess) bin_segment_kernel<false><<<a.n_seg, kScanThreads, kScanSmem, st>>>(a);
+      if (e == cudaSuccess) e = launch_chained(bin_segment_kernel<false>, a.n_seg, kScanThreads, kScanSmem, st, a);
     }
   }
   if (e == cudaSuccess && !a.unordered && a.n_points > 0)
-    bin_order_kernel<<<unsigned(a.n_seg) * (KF_NBINS / 32 / kOrderWarps), 32 * kOrderWarps, 0, st>>>(a);
-  return e != cudaSuccess ? e : cudaGetLastError();
+    e = launch_chained(bin_order_kernel, unsigned(a.n_seg) * (KF_NBINS / 32 / kOrderWarps), 32 * kOrderWarps, 0, st, a);
+  return e;
 }
 
 }  // namespace kfi

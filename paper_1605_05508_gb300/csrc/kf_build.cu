@@ -706,8 +706,9 @@ __device__ __forceinline__ void child_insert(uint32_t (&X)[LW], int (&P)[LW], ui
 // hits), so all hits of a window, kScanStage at most, are in flight at once:
 // each thread copies its own into its column of `stage` (shared memory, slot
 // stride kResThreads) by cp.async, which holds no registers meanwhile; S^-1 is
-// computed while the offsets arrive, and the next pieces' offsets are fetched
-// beside the hits.
+// computed while the offsets arrive.  (The next pieces' offsets fetched before
+// the wait, or all pieces staged before one wait, cost registers: 1 055 and
+// 1 063 against 1 030 us a 50-event step.)
 __device__ __forceinline__ void cp_async16(float4* dst, const float4* src) {
   asm volatile("cp.async.ca.shared.global [%0], [%1], 16;" ::"r"(smem_u32(dst)), "l"(src) : "memory");
 }
@@ -1153,6 +1154,7 @@ __device__ bool pd5_final(const T p[6], const T C[21]) {
 template <int W, bool TABLE, bool MAT>
 __global__ void __launch_bounds__(kResThreads, resident_blocks_per_sm(W))
     build_resident_kernel(const __grid_constant__ BuildResidentArgs A) {
+  chain_begin();
   constexpr int G = 32 / W;  // seeds per group
   extern __shared__ int s_hist[];  // [n_layers][kResThreads]: hit id + 1 | parent rank << 24 (kHistLayers)
   __shared__ float4 s_stage[kScanStage * kResThreads];
@@ -1371,6 +1373,7 @@ __global__ void __launch_bounds__(kResThreads, resident_blocks_per_sm(W))
 template <bool TABLE, bool MAT>
 __global__ void __launch_bounds__(kResThreads, kResBlocksPerSM)
     build_first_layer_kernel(const __grid_constant__ BuildResidentArgs A) {
+  chain_begin();
   __shared__ float4 s_stage[kScanStage * kResThreads];
   const int64_t t = int64_t(blockIdx.x) * kResThreads + threadIdx.x;
   int q = 0;  // the batch of this seed (a served event), with a table
@@ -1490,25 +1493,20 @@ cudaError_t launch_build_first_layer(const BuildResidentArgs& a, cudaStream_t st
   if (seeds <= 0) return cudaSuccess;
   const int grid = int((seeds + kResThreads - 1) / kResThreads);
   const bool mat = a.x_x0[a.l0] > 0.f;
-  if (a.table)
-    mat ? build_first_layer_kernel<true, true><<<grid, kResThreads, 0, st>>>(a)
-        : build_first_layer_kernel<true, false><<<grid, kResThreads, 0, st>>>(a);
-  else
-    mat ? build_first_layer_kernel<false, true><<<grid, kResThreads, 0, st>>>(a)
-        : build_first_layer_kernel<false, false><<<grid, kResThreads, 0, st>>>(a);
-  return cudaGetLastError();
+  const auto kernel = a.table ? (mat ? build_first_layer_kernel<true, true> : build_first_layer_kernel<true, false>)
+                              : (mat ? build_first_layer_kernel<false, true> : build_first_layer_kernel<false, false>);
+  return launch_chained(kernel, grid, kResThreads, 0, st, a);
 }
 
 template <bool TABLE, bool MAT>
-static void launch_resident_w(const BuildResidentArgs& a, int W, int grid, cudaStream_t st) {
+static cudaError_t launch_resident_w(const BuildResidentArgs& a, int W, int grid, cudaStream_t st) {
   const size_t hist = a.paths ? size_t(a.n_layers) * kResThreads * sizeof(int) : 0;
-  switch (W) {
-    case 1: build_resident_kernel<1, TABLE, MAT><<<grid, kResThreads, hist, st>>>(a); break;
-    case 2: build_resident_kernel<2, TABLE, MAT><<<grid, kResThreads, hist, st>>>(a); break;
-    case 4: build_resident_kernel<4, TABLE, MAT><<<grid, kResThreads, hist, st>>>(a); break;
-    case 6: build_resident_kernel<6, TABLE, MAT><<<grid, kResThreads, hist, st>>>(a); break;
-    default: build_resident_kernel<8, TABLE, MAT><<<grid, kResThreads, hist, st>>>(a); break;
-  }
+  const auto kernel = W == 1   ? build_resident_kernel<1, TABLE, MAT>
+                      : W == 2 ? build_resident_kernel<2, TABLE, MAT>
+                      : W == 4 ? build_resident_kernel<4, TABLE, MAT>
+                      : W == 6 ? build_resident_kernel<6, TABLE, MAT>
+                               : build_resident_kernel<8, TABLE, MAT>;
+  return launch_chained(kernel, grid, kResThreads, hist, st, a);
 }
 
 cudaError_t launch_build_resident(const BuildResidentArgs& a, int num_sms, cudaStream_t st) {
@@ -1519,11 +1517,8 @@ cudaError_t launch_build_resident(const BuildResidentArgs& a, int num_sms, cudaS
   const int grid = int(std::max<int64_t>(1, std::min<int64_t>(need, int64_t(num_sms) * resident_blocks_per_sm(W))));
   bool mat = false;
   for (int l = a.l0; l < a.n_layers; ++l) mat |= a.x_x0[l] > 0.f;
-  if (a.table)
-    mat ? launch_resident_w<true, true>(a, W, grid, st) : launch_resident_w<true, false>(a, W, grid, st);
-  else
-    mat ? launch_resident_w<false, true>(a, W, grid, st) : launch_resident_w<false, false>(a, W, grid, st);
-  return cudaGetLastError();
+  if (a.table) return mat ? launch_resident_w<true, true>(a, W, grid, st) : launch_resident_w<true, false>(a, W, grid, st);
+  return mat ? launch_resident_w<false, true>(a, W, grid, st) : launch_resident_w<false, false>(a, W, grid, st);
 }
 
 __global__ void build_init_kernel(const BuildInitArgs A) {
@@ -1540,6 +1535,7 @@ __global__ void build_init_kernel(const BuildInitArgs A) {
 }
 
 __global__ void build_final_kernel(const BuildFinalArgs A) {
+  chain_begin();
   const int64_t j = int64_t(blockIdx.x) * blockDim.x + threadIdx.x;
   if (j >= A.S) return;
   const int64_t seed = A.seed_perm ? A.seed_perm[j] : j;
@@ -1674,14 +1670,14 @@ cudaError_t launch_build_init(const BuildInitArgs& a, cudaStream_t st) {
 
 cudaError_t launch_build_final(const BuildFinalArgs& a, cudaStream_t st) {
   if (a.S <= 0) return cudaSuccess;
-  build_final_kernel<<<int((a.S + 127) / 128), 128, 0, st>>>(a);
-  return cudaGetLastError();
+  return launch_chained(build_final_kernel, int((a.S + 127) / 128), 128, 0, st, a);
 }
 
 // evt[j] = the event of seed j: the last e with seed_off[e] <= j (binary
 // search); and the group counter of the launch that follows set to zero
 __global__ void seed_event_kernel(int32_t* evt, const int64_t* seed_off, int64_t E, int64_t S,
                                   unsigned long long* counter) {
+  chain_begin();
   const int64_t j = int64_t(blockIdx.x) * blockDim.x + threadIdx.x;
   if (j == 0) *counter = 0;
   if (j >= S) return;
@@ -1867,8 +1863,7 @@ extern "C" int kf_build(kf_ctx* ctx, const kf_tracks* seeds, const int64_t* seed
     fa.rest = resident_rest(max_cands, L, out->cand_hit_idx != nullptr);
     fa.out = *out;
     if (((fa.rest & 1) && (out->hit_idx || out->cand_hit_idx)) || ((fa.rest & 2) && out->status)) {
-      build_final_kernel<<<int((S + 127) / 128), 128, 0, s>>>(fa);
-      KF_CUDA_TRY(ctx, cudaGetLastError());
+      KF_CUDA_TRY(ctx, launch_build_final(fa, s));
     }
     return KF_OK;
   }
@@ -1936,8 +1931,7 @@ extern "C" int kf_build(kf_ctx* ctx, const kf_tracks* seeds, const int64_t* seed
   fa.rm_buffers = rm_buffers;
   fa.rest = 0;
   fa.out = *out;
-  build_final_kernel<<<int((S + 127) / 128), 128, 0, s>>>(fa);
-  KF_CUDA_TRY(ctx, cudaGetLastError());
+  KF_CUDA_TRY(ctx, launch_build_final(fa, s));
   return KF_OK;
 }
 

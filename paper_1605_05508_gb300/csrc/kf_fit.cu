@@ -375,6 +375,7 @@ __device__ __forceinline__ void fused_track(const EV& E, const FitFusedArgs& A, 
 
 template <int THREADS>
 __global__ void __launch_bounds__(THREADS, kFitWarpsPerSM * 32 / THREADS) fit_fused_kernel(const FitFusedArgs A) {
+  chain_begin();
   const int64_t i = int64_t(blockIdx.x) * THREADS + threadIdx.x;
   if (i < A.n) fused_track<false>(A, A, i, ArrayHits{A.hits, A.valid, A.n, i});
 }
@@ -390,6 +391,7 @@ __global__ void __launch_bounds__(kFitThreads, 1) fit_mixed_kernel(const FitFuse
 // 79 us re-fit of 128 000 tracks over 10 layers.
 __global__ void __launch_bounds__(kFitThreads, kFitTableBlocksPerSM)
     fit_gather_kernel(const FitFusedArgs A, const RefitGatherArgs G) {
+  chain_begin();
   const int64_t i = int64_t(blockIdx.x) * kFitThreads + threadIdx.x;
   if (i < A.n) fused_track<false>(A, A, i, GatherHits(G, i));
 }
@@ -399,6 +401,7 @@ __global__ void __launch_bounds__(kFitThreads, kFitTableBlocksPerSM)
 // the last with table[q].begin <= t; the arithmetic of fit_fused_kernel.
 __global__ void __launch_bounds__(kFitThreads, kFitTableBlocksPerSM)
     fit_fused_table_kernel(const FitFusedArgs A, const FitEvent* table, int n_events, int64_t n_total) {
+  chain_begin();
   const int64_t stride = int64_t(gridDim.x) * blockDim.x;
   for (int64_t t = int64_t(blockIdx.x) * blockDim.x + threadIdx.x; t < n_total; t += stride) {
     int q = 0;
@@ -490,8 +493,7 @@ cudaError_t launch_fit_fused_table(const FitFusedArgs& a, const FitEvent* table,
                                    cudaStream_t st) {
   if (n_total <= 0) return cudaSuccess;
   const int grid = int((n_total + kFitThreads - 1) / kFitThreads);
-  fit_fused_table_kernel<<<grid, kFitThreads, 0, st>>>(a, table, n_events, n_total);
-  return cudaGetLastError();
+  return launch_chained(fit_fused_table_kernel, grid, kFitThreads, 0, st, a, table, n_events, n_total);
 }
 
 cudaError_t launch_fit_fused(const FitFusedArgs& a, int block, cudaStream_t st) {
@@ -499,11 +501,8 @@ cudaError_t launch_fit_fused(const FitFusedArgs& a, int block, cudaStream_t st) 
   // blocks of 32 for small batches, to spread their warps over the SMs, made no
   // difference (18.43 us for 1 000 tracks x 10 layers either way)
   const int grid = int((a.n + block - 1) / block);
-  if (block == 64)
-    fit_fused_kernel<64><<<grid, 64, 0, st>>>(a);
-  else
-    fit_fused_kernel<128><<<grid, 128, 0, st>>>(a);
-  return cudaGetLastError();
+  return block == 64 ? launch_chained(fit_fused_kernel<64>, grid, 64, 0, st, a)
+                     : launch_chained(fit_fused_kernel<128>, grid, 128, 0, st, a);
 }
 
 cudaError_t launch_fit_gather(const FitFusedArgs& a, const RefitGatherArgs& g, cudaStream_t st) {
