@@ -631,22 +631,22 @@ def build_kernel_name(t, max_cands):
 
 
 def build_step_launches(tune, Lb, max_cands):
-    """Kernel launches of one build step: the seed fit (one), the hit binning (one launch unordered, else count, scan, scatter, sort) and
-    kf_build -- register-resident: the seeds' events, the first layer (with
-    more than one lane a seed), the other layers, the final pass; else the seed
-    ordering (count, scan, scatter), global ids, first candidates, the layer
-    steps and the final selection."""
-    binning = 1 if tune.get("bin_unordered") else 4
+    """Kernel launches of one build step of many segments: the seed fit (one),
+    the hit binning (one block a segment; ordered, the order by id too) and
+    kf_build -- register-resident: with more than one lane a seed the first
+    layer, the other layers and the covariance check, else the seeds' events
+    and the layers; else the seed ordering, global ids, first candidates, the
+    layer steps and the final selection."""
+    binning = 1 if tune.get("bin_unordered") else 2
     if tune["build_scan"] == 4:
-        lanes = max_cands if max_cands <= 2 else 4 if max_cands <= 4 else 6 if max_cands <= 6 else 8
-        build = 1 + (1 if lanes > 1 and Lb > 1 else 0) + 1 + 1
+        build = 3 if max_cands > 1 else 2
     else:
         steps = Lb
         if tune["build_scan"] in (2, 3):  # packed: one launch per layer up to the layout switch, then one
             rm = Lb + 1 if max_cands <= 2 else 2
             first_fused = 0 if rm > Lb else min(Lb, rm)
             steps = first_fused + 1 if first_fused < Lb else Lb
-        build = 3 + 1 + 1 + steps + 1
+        build = 1 + 1 + 1 + steps + 1
     return 1 + binning + build
 
 

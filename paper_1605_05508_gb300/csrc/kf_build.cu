@@ -1022,18 +1022,22 @@ __global__ void __launch_bounds__(NT, kBuildBlocksPerSM * kBuildThreads / NT) bu
 // band of seeds, whose events' hits stay in L2); lane k of a seed's W lanes
 // holds the seed's candidate of rank k.  Per building layer, every live lane
 // propagates its candidate, derives the window and scans it into a sorted
-// list of its best children's keys;
-// the seed's lanes merge their lists by a minimum over the seed's lanes of the
-// 64-bit keys (full-warp shuffles rotating within each seed's lanes) into
-// the seed's best max_cands, ranked by the same total order; lane k then
-// pulls the predicted state and S^-1 of its winner's parent from that lane by
-// shuffles and applies the Kalman update with the winner's hit.  Only the
-// per-layer history (parent rank, hit id) goes to memory; after the last
-// layer the best candidates are written to the caller's result (or every
-// candidate to the last buffer, for a final selection).  Groups are
-// independent, so warps run at their own pace (no block barrier).  The keys
-// are a total order and every candidate goes through the same functions as in
-// the other layouts, so the results are bitwise theirs.
+// list of its best children (child_insert); the children of the seed's lanes
+// are ranked by the same total order as the keys' by counting over rotating
+// shuffles (merge_children); lane k then pulls the predicted state and S^-1 of
+// its winner's parent from that lane by shuffles and applies the Kalman update
+// with the winner's hit.  The history (parent rank, hit id) stays in shared
+// memory, and after the last layer the best candidates and their paths are
+// written to the caller's result.  Groups are independent, so warps run at
+// their own pace (no block barrier).  The order is total and every candidate
+// goes through the same functions as in the other layouts, so the results are
+// bitwise theirs.
+//
+// What bounds it, of 10 events x 5 000 seeds (ncu): instruction issue (68 % of
+// the cycles, 129 M warp instructions with 17.5 of 32 lanes active: a seed owns
+// W lanes whatever it holds), instruction fetch (45 KB of code) and the
+// dependent loads of the windows; 167 us, where the 64-bit-key form with
+// direct loads took 249 us (56 %, 165 M).
 
 // The kept children of a seed, one per lane: lane k of the seed's W lanes
 // (lanes gbase .. gbase + W - 1, mask seg) receives the k-th best.
