@@ -219,11 +219,11 @@ typedef struct {
 } kf_layer_hit_bins;
 
 /* Sort every segment's hits into the eta x phi bins (Sec. 3: hits sorted in
- * phi within eta bins per layer, phi bins for fast look-up): a counting sort
- * over all segments at once (count, per-segment scan, scatter, then an id
- * sort inside each bin, so the order is deterministic), or with
- * kf_tuning.bin_unordered one block per segment and no id sort (with
- * `out->fine_off` set: by sub-bin, and the sub-bin starts written too).
+ * phi within eta bins per layer, phi bins for fast look-up): a counting sort,
+ * by passes over all segments' hits at once or by one block per segment
+ * (chosen by their mean size), then a pass that orders each bin by id, so the
+ * order is deterministic, or with kf_tuning.bin_unordered without that pass
+ * (with `out->fine_off` set: by sub-bin, and the sub-bin starts written too).
  * `out->hits`, `out->bin_off` (and `out->fine_off`) are caller-allocated with
  * the sizes above; the other fields of `out` are set from `in`.  Segments must hold at most KF_MAX_HITS_PER_SEGMENT hits (not
  * checked here: seg_off is device memory; kf_build ignores hits beyond it).
