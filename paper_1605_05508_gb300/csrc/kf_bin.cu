@@ -300,43 +300,136 @@ __global__ void __launch_bounds__(kPointThreads) bin_place_kernel(const BinArgs 
   S.out_pts[S.p0 + at] = make_float4(x, y, z, __int_as_float(int(q - S.p0)));
 }
 
-// One warp per 32 bins of a segment: their hits, ids in any order inside a
-// bin, are a contiguous run.  Runs of up to kOrderRun hits are taken whole:
-// loaded (coalesced, all in flight), every hit's place found by counting the
-// smaller ids of its bin in shared memory, and the moved ones written back.
-// Of a longer run, as many bins as fit are taken at a time; a single bin that
-// does not fit is sorted by one insertion sort.
+// One warp per NB bins of a segment: their hits, ids in any order inside a bin,
+// are a contiguous run.  Runs of up to kOrderRun hits are taken whole: loaded
+// (coalesced, all in flight), every hit's place found by counting the smaller
+// ids of its bin in shared memory, and the moved ones written back.  Of a
+// longer run, as many bins as fit are taken at a time; a single bin that does
+// not fit goes through order_long_bin, after the others.
 constexpr int kOrderRun = 128;
 constexpr int kOrderWarps = 4;
-__global__ void __launch_bounds__(32 * kOrderWarps) bin_order_kernel(const BinArgs A) {
+
+// A bin of more than kOrderRun hits, n from `beg` of segment s on, by one warp:
+// a radix sort of the ids (stable passes of 7 bits, the counters in shared
+// memory, between out_pts[].w and the bin's part of the scratch out_id, whose
+// words the passes before are done with), after which every hit is fetched by
+// its id.  The time is linear in n: 60 000 hits in some 325 bins take 88 us,
+// 5 000 in 25 bins 65; by one lane's insertion sort, the bins of a warp one
+// after the other, 5.6 and 9.6 ms, by one a thread a bin 1.1 and 1.7 ms.
+constexpr int kDigitBits = 7;
+__device__ __forceinline__ void order_long_bin(const BinArgs& A, int s, int beg, int n, int* digits) {
+  const int64_t p0 = A.seg_off[s], m = min(A.seg_off[s + 1], A.stride) - p0;
+  float4* const pts = A.out_pts + p0 + beg;
+  int* const tmp = A.out_id + p0 + beg;
+  constexpr int kDigits = 1 << kDigitBits, kAhead = 4;  // ids a lane has in flight
+  const int lane = threadIdx.x & 31;
+  bool in_tmp = false;  // where the ids are
+  for (int shift = 0; shift < 31 && (m - 1) >> shift > 0; shift += kDigitBits) {
+    for (int t = lane; t < kDigits; t += 32) digits[t] = 0;
+    __syncwarp();
+    auto load = [&](int i0, int (&id)[kAhead]) {
+#pragma unroll
+      for (int t = 0; t < kAhead; ++t) {
+        const int i = i0 + 32 * t + lane;
+        id[t] = i < n ? (in_tmp ? tmp[i] : __float_as_int(pts[i].w)) : -1;
+      }
+    };
+    for (int i0 = 0; i0 < n; i0 += 32 * kAhead) {
+      int id[kAhead];
+      load(i0, id);
+#pragma unroll
+      for (int t = 0; t < kAhead; ++t)
+        if (id[t] >= 0) atomicAdd(&digits[(id[t] >> shift) & (kDigits - 1)], 1);
+    }
+    __syncwarp();
+    {  // counts to starts, kDigits / 32 of them a lane
+      constexpr int kPer = kDigits / 32;
+      int v[kPer], sum = 0;
+#pragma unroll
+      for (int t = 0; t < kPer; ++t) {
+        v[t] = digits[lane * kPer + t];
+        sum += v[t];
+      }
+      int inc = sum;
+#pragma unroll
+      for (int d = 1; d < 32; d *= 2) {
+        const int o = __shfl_up_sync(0xffffffffu, inc, d);
+        if (lane >= d) inc += o;
+      }
+      int at = inc - sum;
+#pragma unroll
+      for (int t = 0; t < kPer; ++t) {
+        digits[lane * kPer + t] = at;
+        at += v[t];
+      }
+    }
+    __syncwarp();
+    for (int i0 = 0; i0 < n; i0 += 32 * kAhead) {
+      int id[kAhead];
+      load(i0, id);
+#pragma unroll
+      for (int t = 0; t < kAhead; ++t) {
+        const int d = id[t] >= 0 ? (id[t] >> shift) & (kDigits - 1) : kDigits;
+        const unsigned same = __match_any_sync(0xffffffffu, d);
+        const int before = __popc(same & ((1u << lane) - 1u));
+        int at = 0;
+        if (id[t] >= 0) at = digits[d] + before;
+        __syncwarp();
+        if (id[t] >= 0) {
+          if (before == 0) digits[d] += __popc(same);
+          if (in_tmp)
+            pts[at].w = __int_as_float(id[t]);
+          else
+            tmp[at] = id[t];
+        }
+        __syncwarp();
+      }
+    }
+    in_tmp = !in_tmp;
+  }
+  for (int i = lane; i < n; i += 32) {
+    const int id = in_tmp ? tmp[i] : __float_as_int(pts[i].w);
+    const float* const h = A.xyz + p0 + id;
+    pts[i] = make_float4(h[0], h[A.stride], h[2 * A.stride], __int_as_float(id));
+  }
+  __syncwarp();  // the counters are free again
+}
+
+// (10 or 11 blocks an SM, as measured: with 10 one segment of 1 500 000 hits takes
+// 140 us, not 165, with 11 350 of 20 000 202, not 206)
+template <int NB>
+__global__ void __launch_bounds__(32 * kOrderWarps, NB <= 8 ? 10 : 11) bin_order_kernel(const __grid_constant__ BinArgs A) {
   chain_begin();
   __shared__ int s_id[kOrderWarps][kOrderRun];
-  __shared__ int s_off[kOrderWarps][33];
+  __shared__ int s_off[kOrderWarps][NB + 1];
+  static_assert(kOrderRun >= 1 << kDigitBits, "s_id holds order_long_bin's counters");
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   int* const ids = s_id[warp];
   int* const off = s_off[warp];
-  const int s = int(blockIdx.x) / (KF_NBINS / 32 / kOrderWarps);
-  const int b0 = (int(blockIdx.x) % (KF_NBINS / 32 / kOrderWarps) * kOrderWarps + warp) * 32;
+  const int s = int(blockIdx.x) / (KF_NBINS / NB / kOrderWarps);
+  const int b0 = (int(blockIdx.x) % (KF_NBINS / NB / kOrderWarps) * kOrderWarps + warp) * NB;
   const int32_t* const starts = A.bin_off + int64_t(s) * (KF_NBINS + 1) + b0;
   float4* const pts = A.out_pts + A.seg_off[s];
-  const int mine = starts[lane];
-  off[lane] = mine;
-  if (lane == 0) off[32] = starts[32];
+#pragma unroll
+  for (int b = lane; b <= NB; b += 32) off[b] = starts[b];
   __syncwarp();
-  const int end_all = off[32];
-  for (int bb = 0; bb < 32 && off[bb] < end_all;) {
+  const int end_all = off[NB];
+  bool crowded = false;
+  for (int bb = 0; bb < NB && off[bb] < end_all;) {
     const int beg = off[bb];
     // the bins bb .. be-1 whose hits fit a run
-    int be = 33 - __popc(__ballot_sync(0xffffffffu, off[lane + 1] - beg > kOrderRun && lane >= bb)) - 1;
-    if (be == bb) {  // one bin alone is too long
-      if (lane == 0)
-        for (int u = beg + 1; u < off[bb + 1]; ++u) {
-          const float4 pt = pts[u];
-          int v = u - 1;
-          for (; v >= beg && __float_as_int(pts[v].w) > __float_as_int(pt.w); --v) pts[v + 1] = pts[v];
-          pts[v + 1] = pt;
-        }
-      bb = be + 1;
+    int be = bb, above = NB + 1;
+    if (end_all - beg <= kOrderRun) be = NB;
+    while (above - be > 1) {
+      const int mid = (be + above) >> 1;
+      if (off[mid] - beg <= kOrderRun)
+        be = mid;
+      else
+        above = mid;
+    }
+    if (be == bb) {  // one bin alone is too long: below
+      crowded = true;
+      ++bb;
       continue;
     }
     const int n = off[be] - beg;
@@ -369,6 +462,9 @@ __global__ void __launch_bounds__(32 * kOrderWarps) bin_order_kernel(const BinAr
     __syncwarp();  // ids are read before the next run's
     bb = be;
   }
+  if (crowded)
+    for (int b = 0; b < NB; ++b)
+      if (off[b + 1] - off[b] > kOrderRun) order_long_bin(A, s, off[b], off[b + 1] - off[b], ids);
 }
 
 constexpr int kMaxDevices = 64;
@@ -416,6 +512,27 @@ cudaError_t launch_bin_segment_table(const BinSegment* table, int n, int64_t n_p
   return fine ? launch_bin_wide<true>(a, st) : launch_bin_wide<false>(a, st);
 }
 
+// Bins a warp of the order pass takes.  A warp's runs follow one another, and
+// a warp of few hits costs its launch and its loads all the same, so: about as
+// many bins as hold one run at the mean density, as long as every SM has some
+// twenty warps.  After the wide passes, whose segments may be of very different
+// sizes, no more than 32.  Whole binning, measured with 128, 64, 32 and 8 bins
+// a warp: 350 segments of 20 000 hits 207, 202, 227 and 418 us, 1 540 of 1 000
+// 124, -, 283 and 861; 7 of 20 000 26.8, -, 21.6 and 23.7; one of 1 500 000
+// 1 456, -, 405 and 140.
+static cudaError_t launch_bin_order(const BinArgs& a, int num_sms, bool wide, cudaStream_t st) {
+  const auto go = [&](void (*kernel)(BinArgs), int nb) {
+    return launch_chained(kernel, unsigned(a.n_seg) * unsigned(KF_NBINS / nb / kOrderWarps), 32 * kOrderWarps, 0, st,
+                          a);
+  };
+  const auto fills = [&](int nb) { return int64_t(a.n_seg) * (KF_NBINS / nb) >= int64_t(num_sms) * 20; };
+  const auto one_run = [&](int nb) { return a.n_points * nb <= int64_t(a.n_seg) * kOrderRun * KF_NBINS; };
+  if (!wide && fills(128) && one_run(128)) return go(bin_order_kernel<128>, 128);
+  if (!wide && fills(64) && one_run(64)) return go(bin_order_kernel<64>, 64);
+  if (fills(32)) return go(bin_order_kernel<32>, 32);
+  return go(bin_order_kernel<8>, 8);
+}
+
 // Which form: one block per segment costs about 10 us plus 1.3 us per 1 000
 // hits of the largest segment, times the rounds of segments on the SMs; the
 // wide passes 20 us plus 0.024 us per 1 000 hits of all segments (measured:
@@ -432,7 +549,8 @@ cudaError_t launch_bin_points(const BinArgs& a, int num_sms, cudaStream_t st) {
   if (a.n_seg <= 0) return cudaSuccess;
   if (a.fine_off && !a.unordered) return cudaErrorInvalidValue;  // sub-bins only with the unordered binning
   cudaError_t e;
-  if (!one_block_a_segment(a, num_sms)) {
+  const bool wide = !one_block_a_segment(a, num_sms);
+  if (wide) {
     e = a.fine_off ? launch_bin_wide<true>(a, st) : launch_bin_wide<false>(a, st);
   } else {
     static std::atomic<bool> seg_attr_set[kMaxDevices], fine_attr_set[kMaxDevices];
@@ -445,7 +563,7 @@ cudaError_t launch_bin_points(const BinArgs& a, int num_sms, cudaStream_t st) {
     }
   }
   if (e == cudaSuccess && !a.unordered && a.n_points > 0)
-    e = launch_chained(bin_order_kernel, unsigned(a.n_seg) * (KF_NBINS / 32 / kOrderWarps), 32 * kOrderWarps, 0, st, a);
+    e = launch_bin_order(a, num_sms, wide, st);
   return e;
 }
 
