@@ -221,7 +221,8 @@ typedef struct {
 /* Sort every segment's hits into the eta x phi bins (Sec. 3: hits sorted in
  * phi within eta bins per layer, phi bins for fast look-up): a counting sort,
  * by passes over all segments' hits at once or by one block per segment
- * (chosen by their mean size), then a pass that orders each bin by id, so the
+ * (chosen by their mean size; in the ordered form segments far beyond it go by
+ * passes all the same), then a pass that orders each bin by id, so the
  * order is deterministic, or with kf_tuning.bin_unordered without that pass
  * (with `out->fine_off` set: by sub-bin, and the sub-bin starts written too).
  * `out->hits`, `out->bin_off` (and `out->fine_off`) are caller-allocated with

@@ -15,12 +15,14 @@
 
 #include <algorithm>
 #include <atomic>
+#include <limits>
 
 namespace kfi {
 
 constexpr int kScanThreads = 1024;
 static_assert(KF_NBINS % kScanThreads == 0, "bins per thread");  // 16 consecutive bins a thread
 constexpr int kPointThreads = 256;
+constexpr int64_t kNoLimit = std::numeric_limits<int64_t>::max();  // of a segment's points
 
 // padded shared-memory index of bin b: a thread's 16 (or 32) consecutive
 // bins and a warp's 32 threads fall in distinct banks
@@ -72,6 +74,35 @@ __device__ __forceinline__ int scan_bins(int* cnt, int* warp_tot) {
   return total;
 }
 
+// segment s of the request: a table entry, or segment s of the arrays of A
+template <bool FINE>
+__device__ __forceinline__ BinSegment segment(const BinArgs& A, int s) {
+  if (A.table) return A.table[s];
+  BinSegment S;
+  S.xyz = A.xyz;
+  S.stride = A.stride;
+  S.p0 = A.seg_off[s];
+  S.p1 = min(A.seg_off[s + 1], A.stride);
+  S.begin = S.p0;
+  S.bin_off = A.bin_off + int64_t(s) * (KF_NBINS + 1);
+  S.fine_off = FINE ? A.fine_off + int64_t(s) * (KF_NBINS_FINE + 1) : nullptr;
+  S.out_pts = A.out_pts;
+  S.out_id = A.out_id;
+  return S;
+}
+// the last segment that begins at or before point g of the launch's points
+__device__ __forceinline__ int segment_of(const BinArgs& A, int64_t g) {
+  int lo = 0, hi = A.n_seg - 1;
+  while (lo < hi) {
+    const int mid = (lo + hi + 1) >> 1;
+    if ((A.table ? A.table[mid].begin : A.seg_off[mid]) <= g)
+      lo = mid;
+    else
+      hi = mid - 1;
+  }
+  return lo;
+}
+
 // The unordered counting sort of one segment per block, its counts and
 // cursors in shared memory (one launch for all segments): (1) every point of
 // the segment adds one to its bin's count, (2) the block turns the counts
@@ -79,15 +110,20 @@ __device__ __forceinline__ int scan_bins(int* cnt, int* warp_tot) {
 // takes the next slot of its bin.  The order inside a bin is that of the
 // shared-memory atomics: for kf_tuning.bin_unordered, whose users do not
 // depend on it.
-// The points [p0, p1) of xyz ([3][stride]) of one segment, by the whole
-// block, with cnt (KF_NBINS padded ints of shared memory) and warp_tot.
+// Segment S (number seg) by the whole block, with cnt (KF_NBINS padded ints of
+// shared memory) and warp_tot.
 // FINE: the counting sort runs over the KF_NBINS_FINE sub-bins (cnt holds
 // as many), whose starts go to fine_off, and the bin starts to `off` are
 // those of the even sub-bins (a bin is two consecutive sub-bins).
 template <bool FINE = false>
-__device__ __forceinline__ void bin_one_segment(const float* xyz, int64_t stride, int64_t p0, int64_t p1,
-                                                int32_t* off, int32_t* fine_off, float4* out_pts, int32_t* out_id,
-                                                int32_t* out_seg, int seg, int* cnt, int* warp_tot) {
+__device__ __forceinline__ void bin_one_segment(const BinSegment& S, int32_t* out_seg, int seg, int* cnt,
+                                                int* warp_tot) {
+  const float* const xyz = S.xyz;
+  const int64_t stride = S.stride, p0 = S.p0, p1 = S.p1;
+  int32_t* const off = S.bin_off;
+  int32_t* const fine_off = S.fine_off;
+  float4* const out_pts = S.out_pts;
+  int32_t* const out_id = S.out_id;
   constexpr int NB = FINE ? KF_NBINS_FINE : KF_NBINS;
   constexpr int NPHI = FINE ? KF_BIN_PHI_FINE : KF_BIN_PHI;
   const int tid = threadIdx.x;
@@ -162,16 +198,18 @@ __device__ __forceinline__ void bin_one_segment(const float* xyz, int64_t stride
   }
 }
 
+// (a segment of more than `limit` points is left to bin_large_count_kernel and
+// what follows it, its counts set to zero)
 template <bool FINE>
-__global__ void __launch_bounds__(kScanThreads) bin_segment_kernel(const BinArgs A) {
+__global__ void __launch_bounds__(kScanThreads) bin_segment_kernel(const BinArgs A, const int64_t limit) {
   chain_begin();
   extern __shared__ int cnt[];  // counts, then cursors (padded layout)
   __shared__ int warp_tot[32];
-  const int seg = blockIdx.x;
-  bin_one_segment<FINE>(A.xyz, A.stride, A.seg_off[seg], min(A.seg_off[seg + 1], A.stride),
-                        A.bin_off + int64_t(seg) * (KF_NBINS + 1),
-                        FINE ? A.fine_off + int64_t(seg) * (KF_NBINS_FINE + 1) : nullptr, A.out_pts, A.out_id,
-                        A.out_seg, seg, cnt, warp_tot);
+  const BinSegment S = segment<FINE>(A, int(blockIdx.x));
+  if (S.p1 - S.p0 <= limit)
+    bin_one_segment<FINE>(S, A.out_seg, int(blockIdx.x), cnt, warp_tot);
+  else if (!FINE)
+    for (int b = threadIdx.x; b <= KF_NBINS; b += kScanThreads) S.bin_off[b] = 0;
 }
 
 // ---------------------------------------------------------------------------
@@ -182,8 +220,8 @@ __global__ void __launch_bounds__(kScanThreads) bin_segment_kernel(const BinArgs
 //                     it is its place in the bin, kept with the bin in one word
 //   bin_scan_kernel   one block per segment: counts to starts
 //   bin_place_kernel  every point to its bin's start plus its place
-//   bin_order_kernel  (ordered form) a warp sorts the hits of 32 consecutive
-//                     bins, a contiguous run, by id inside each bin
+//   bin_order_kernel  (ordered form) a warp sorts the hits of consecutive bins,
+//                     a contiguous run, by id inside each bin
 // A point's word between the passes: its bin above its place, or, with the top
 // bit set, its position in the segment.  A place of kPlaceMax or more (a bin of
 // more than 65 535 hits) does not fit: the count leaves it in the point's own
@@ -193,35 +231,6 @@ constexpr int kPlaceBits = 16;
 constexpr uint32_t kPlaceMax = (1u << kPlaceBits) - 1;
 constexpr uint32_t kIsPosition = 1u << 31;
 static_assert(KF_NBINS_FINE <= 1 << (31 - kPlaceBits), "bin and place in a word");
-
-// segment s of the request: a table entry, or segment s of the arrays of A
-template <bool FINE>
-__device__ __forceinline__ BinSegment segment(const BinArgs& A, int s) {
-  if (A.table) return A.table[s];
-  BinSegment S;
-  S.xyz = A.xyz;
-  S.stride = A.stride;
-  S.p0 = A.seg_off[s];
-  S.p1 = min(A.seg_off[s + 1], A.stride);
-  S.begin = S.p0;
-  S.bin_off = A.bin_off + int64_t(s) * (KF_NBINS + 1);
-  S.fine_off = FINE ? A.fine_off + int64_t(s) * (KF_NBINS_FINE + 1) : nullptr;
-  S.out_pts = A.out_pts;
-  S.out_id = A.out_id;
-  return S;
-}
-// the last segment that begins at or before point g of the launch's points
-__device__ __forceinline__ int segment_of(const BinArgs& A, int64_t g) {
-  int lo = 0, hi = A.n_seg - 1;
-  while (lo < hi) {
-    const int mid = (lo + hi + 1) >> 1;
-    if ((A.table ? A.table[mid].begin : A.seg_off[mid]) <= g)
-      lo = mid;
-    else
-      hi = mid - 1;
-  }
-  return lo;
-}
 
 // kZeroPer bins a thread: with one, the launch of the blocks, about one a
 // nanosecond, set the time (21.6 us for the sub-bins of 151 segments; of 151
@@ -238,6 +247,57 @@ __global__ void __launch_bounds__(kPointThreads) bin_zero_kernel(const BinArgs A
   for (int t = 0; t < kZeroPer; ++t) c[t * kPointThreads + threadIdx.x] = 0;
 }
 
+// N points of segment S, q, q + step, .. (those below S.p1), their loads and
+// atomics in flight together
+template <bool FINE, int N>
+__device__ __forceinline__ void count_points(const BinSegment& S, int64_t q, int64_t step) {
+  float x[N], y[N], z[N];
+  uint32_t place[N];
+  int b[N];
+#pragma unroll
+  for (int t = 0; t < N; ++t)
+    if (q + t * step < S.p1) {
+      x[t] = S.xyz[q + t * step];
+      y[t] = S.xyz[S.stride + q + t * step];
+      z[t] = S.xyz[2 * S.stride + q + t * step];
+    }
+#pragma unroll
+  for (int t = 0; t < N; ++t)
+    if (q + t * step < S.p1) {
+      b[t] = bin_of<FINE ? KF_BIN_PHI_FINE : KF_BIN_PHI>(x[t], y[t], z[t]);
+      place[t] = uint32_t(atomicAdd((FINE ? S.fine_off : S.bin_off) + b[t], 1));
+    }
+#pragma unroll
+  for (int t = 0; t < N; ++t)
+    if (q + t * step < S.p1) {
+      if (place[t] >= kPlaceMax) S.out_pts[q + t * step].x = __uint_as_float(place[t]);
+      S.out_id[q + t * step] = int(uint32_t(b[t]) << kPlaceBits | min(place[t], kPlaceMax));
+    }
+}
+template <bool FINE, int N>
+__device__ __forceinline__ void place_points(const BinSegment& S, int64_t q, int64_t step) {
+  float x[N], y[N], z[N];
+  uint32_t w[N];
+#pragma unroll
+  for (int t = 0; t < N; ++t)
+    if (q + t * step < S.p1) {
+      w[t] = uint32_t(S.out_id[q + t * step]);
+      x[t] = S.xyz[q + t * step];
+      y[t] = S.xyz[S.stride + q + t * step];
+      z[t] = S.xyz[2 * S.stride + q + t * step];
+    }
+  int at[N];
+#pragma unroll
+  for (int t = 0; t < N; ++t)
+    if (q + t * step < S.p1)
+      at[t] = w[t] & kIsPosition ? int(w[t] & ~kIsPosition)
+                                 : (FINE ? S.fine_off : S.bin_off)[w[t] >> kPlaceBits] + int(w[t] & kPlaceMax);
+#pragma unroll
+  for (int t = 0; t < N; ++t)
+    if (q + t * step < S.p1)
+      S.out_pts[S.p0 + at[t]] = make_float4(x[t], y[t], z[t], __int_as_float(int(q + t * step - S.p0)));
+}
+
 template <bool FINE>
 __global__ void __launch_bounds__(kPointThreads) bin_count_kernel(const BinArgs A) {
   chain_begin();
@@ -245,21 +305,15 @@ __global__ void __launch_bounds__(kPointThreads) bin_count_kernel(const BinArgs 
   if (g >= A.n_points) return;
   const BinSegment S = segment<FINE>(A, segment_of(A, g));
   const int64_t q = g - S.begin + S.p0;
-  if (q < S.p0 || q >= S.p1) return;  // outside every segment
-  const int b = bin_of<FINE ? KF_BIN_PHI_FINE : KF_BIN_PHI>(S.xyz[q], S.xyz[S.stride + q], S.xyz[2 * S.stride + q]);
-  const uint32_t place = uint32_t(atomicAdd((FINE ? S.fine_off : S.bin_off) + b, 1));
-  if (place >= kPlaceMax) S.out_pts[q].x = __uint_as_float(place);
-  S.out_id[q] = int(uint32_t(b) << kPlaceBits | min(place, kPlaceMax));
+  if (q >= S.p0 && q < S.p1) count_points<FINE, 1>(S, q, 0);  // (else outside every segment)
 }
 
+// Counts of segment S to starts, by the whole block, with cnt (padded) and
+// warp_tot in shared memory.
 template <bool FINE>
-__global__ void __launch_bounds__(kScanThreads) bin_scan_kernel(const BinArgs A) {
-  chain_begin();
+__device__ __forceinline__ void scan_segment(const BinSegment& S, int* cnt, int* warp_tot) {
   constexpr int NB = FINE ? KF_NBINS_FINE : KF_NBINS;
   constexpr int kPer = NB / kScanThreads;
-  extern __shared__ int cnt[];  // counts, then starts (padded layout)
-  __shared__ int warp_tot[32];
-  const BinSegment S = segment<FINE>(A, int(blockIdx.x));
   int32_t* const c = FINE ? S.fine_off : S.bin_off;
   const int tid = threadIdx.x;
   // 16 loads a thread in flight together (coalesced): one after the other they
@@ -287,9 +341,17 @@ __global__ void __launch_bounds__(kScanThreads) bin_scan_kernel(const BinArgs A)
   if (over)
     for (int64_t q = S.p0 + tid; q < S.p1; q += kScanThreads) {
       const uint32_t w = uint32_t(S.out_id[q]);
-      if ((w & kPlaceMax) == kPlaceMax)
-        S.out_id[q] = int(kIsPosition | (uint32_t(cnt[pad_idx(int(w >> kPlaceBits))]) + __float_as_uint(S.out_pts[q].x)));
+      if ((w & kPlaceMax) != kPlaceMax) continue;
+      const uint32_t at = uint32_t(cnt[pad_idx(int(w >> kPlaceBits))]) + __float_as_uint(S.out_pts[q].x);
+      S.out_id[q] = int(kIsPosition | at);
     }
+}
+template <bool FINE>
+__global__ void __launch_bounds__(kScanThreads) bin_scan_kernel(const BinArgs A) {
+  chain_begin();
+  extern __shared__ int cnt[];  // counts, then starts (padded layout)
+  __shared__ int warp_tot[32];
+  scan_segment<FINE>(segment<FINE>(A, int(blockIdx.x)), cnt, warp_tot);
 }
 
 template <bool FINE>
@@ -299,12 +361,7 @@ __global__ void __launch_bounds__(kPointThreads) bin_place_kernel(const BinArgs 
   if (g >= A.n_points) return;
   const BinSegment S = segment<FINE>(A, segment_of(A, g));
   const int64_t q = g - S.begin + S.p0;
-  if (q < S.p0 || q >= S.p1) return;
-  const float x = S.xyz[q], y = S.xyz[S.stride + q], z = S.xyz[2 * S.stride + q];
-  const uint32_t w = uint32_t(S.out_id[q]);
-  const int at = w & kIsPosition ? int(w & ~kIsPosition)
-                                 : (FINE ? S.fine_off : S.bin_off)[w >> kPlaceBits] + int(w & kPlaceMax);
-  S.out_pts[S.p0 + at] = make_float4(x, y, z, __int_as_float(int(q - S.p0)));
+  if (q >= S.p0 && q < S.p1) place_points<FINE, 1>(S, q, 0);
 }
 
 // One warp per NB bins of a segment: their hits, ids in any order inside a bin,
@@ -402,24 +459,19 @@ __device__ __forceinline__ void order_long_bin(const BinArgs& A, int s, int beg,
   __syncwarp();  // the counters are free again
 }
 
-// (10 or 11 blocks an SM, as measured: with 10 one segment of 1 500 000 hits takes
-// 140 us, not 165, with 11 350 of 20 000 202, not 206)
-template <int NB>
-__global__ void __launch_bounds__(32 * kOrderWarps, NB <= 8 ? 10 : 11) bin_order_kernel(const __grid_constant__ BinArgs A) {
-  chain_begin();
-  __shared__ int s_id[kOrderWarps][kOrderRun];
-  __shared__ int s_off[kOrderWarps][NB + 1];
-  static_assert(kOrderRun >= 1 << kDigitBits, "s_id holds order_long_bin's counters");
-  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-  int* const ids = s_id[warp];
-  int* const off = s_off[warp];
-  const int s = int(blockIdx.x) / (KF_NBINS / NB / kOrderWarps);
-  const int b0 = (int(blockIdx.x) % (KF_NBINS / NB / kOrderWarps) * kOrderWarps + warp) * NB;
+// NB bins of segment s from b0 on, by one warp, with ids (kOrderRun) and off (NB
+// + 1) in shared memory; LIMIT: unless the segment has more than `limit` hits.
+template <int NB, bool LIMIT>
+__device__ __forceinline__ void order_bins(const BinArgs& A, int s, int64_t limit, int b0, int* ids, int* off) {
+  static_assert(kOrderRun >= 1 << kDigitBits, "ids holds order_long_bin's counters");
+  const int lane = threadIdx.x & 31;
   const int32_t* const starts = A.bin_off + int64_t(s) * (KF_NBINS + 1) + b0;
-  float4* const pts = A.out_pts + A.seg_off[s];
+  const int64_t p0 = A.seg_off[s], p1 = LIMIT ? A.seg_off[s + 1] : 0;
+  float4* const pts = A.out_pts + p0;
 #pragma unroll
   for (int b = lane; b <= NB; b += 32) off[b] = starts[b];
   __syncwarp();
+  if (LIMIT && p1 - p0 > limit) return;
   const int end_all = off[NB];
   bool crowded = false;
   for (int bb = 0; bb < NB && off[bb] < end_all;) {
@@ -474,6 +526,162 @@ __global__ void __launch_bounds__(32 * kOrderWarps, NB <= 8 ? 10 : 11) bin_order
       if (off[b + 1] - off[b] > kOrderRun) order_long_bin(A, s, off[b], off[b + 1] - off[b], ids);
 }
 
+// (10 or 11 blocks an SM, as measured: with 10 one segment of 1 500 000 hits takes
+// 140 us, not 165, with 11 350 of 20 000 202, not 206; segments of more than
+// `limit` hits are left to bin_large_order_kernel)
+template <int NB, bool LIMIT>
+__global__ void __launch_bounds__(32 * kOrderWarps, NB <= 8 ? 10 : 11)
+    bin_order_kernel(const __grid_constant__ BinArgs A, const int64_t limit) {
+  chain_begin();
+  __shared__ int s_id[kOrderWarps][kOrderRun];
+  __shared__ int s_off[kOrderWarps][NB + 1];
+  const int warp = threadIdx.x >> 5;
+  const int s = int(blockIdx.x) / (KF_NBINS / NB / kOrderWarps);
+  const int b0 = (int(blockIdx.x) % (KF_NBINS / NB / kOrderWarps) * kOrderWarps + warp) * NB;
+  order_bins<NB, LIMIT>(A, s, limit, b0, s_id[warp], s_off[warp]);
+}
+
+// The segments of more than `limit` points of an ordered request whose others
+// take a block each: their counts are zeroed by their blocks, then the passes
+// above run over their points alone, in three launches.  They cost a request
+// without such segments, which the host cannot tell from one with them, 3 to 5
+// us.
+constexpr int kLargePer = 4;  // points a thread has in flight
+constexpr int kLargeUnit = kPointThreads * kLargePer;
+
+// f(s, S, u) for every large segment S (number s), u running over this block's
+// share of its units_of(points) units; then done(S, n, units), n the units taken,
+// if any.
+template <int THREADS, class U, class F, class D>
+__device__ __forceinline__ void for_large(const BinArgs& A, int64_t limit, U units_of, F f, D done) {
+  constexpr int kAhead = 4, kWords = kAhead * THREADS / 32;  // sizes a thread has in flight
+  __shared__ unsigned s_large[kWords];
+  const int tid = threadIdx.x;
+  int64_t u = blockIdx.x;  // this block's next unit, counted on from segment to segment
+  for (int s0 = 0; s0 < A.n_seg; s0 += kAhead * THREADS) {
+    bool any = false, large[kAhead];
+#pragma unroll
+    for (int t = 0; t < kAhead; ++t) {
+      const int s = s0 + t * THREADS + tid;
+      large[t] = s < A.n_seg && min(A.seg_off[s + 1], A.stride) - A.seg_off[s] > limit;
+    }
+#pragma unroll
+    for (int t = 0; t < kAhead; ++t) {
+      const unsigned m = __ballot_sync(0xffffffffu, large[t]);
+      if ((tid & 31) == 0) s_large[(t * THREADS + tid) >> 5] = m;
+      any |= large[t];
+    }
+    if (__syncthreads_or(any))
+      for (int w = 0; w < kWords; ++w)
+        for (unsigned left = s_large[w]; left; left &= left - 1) {
+          const int s = s0 + 32 * w + __ffs(left) - 1;
+          const BinSegment S = segment<false>(A, s);
+          const int64_t units = units_of(S.p1 - S.p0);
+          int n = 0;
+          for (; u < units; u += gridDim.x, ++n) f(s, S, u);
+          u -= units;
+          if (n > 0) done(S, n, int(units));
+        }
+    __syncthreads();  // s_large is read before the next segments'
+  }
+}
+
+// Count; the block that ends a segment's last unit turns the counts to starts
+// (the units done so far are counted in the place of the total).
+__global__ void __launch_bounds__(kPointThreads)
+    bin_large_count_kernel(const __grid_constant__ BinArgs A, const int64_t limit) {
+  chain_begin();
+  __shared__ int s_sum[kPointThreads / 32];
+  __shared__ int s_done;
+  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+  for_large<kPointThreads>(
+      A, limit, [](int64_t points) { return (points + kLargeUnit - 1) / kLargeUnit; },
+      [&](int, const BinSegment& S, int64_t u) {
+        count_points<false, kLargePer>(S, S.p0 + u * kLargeUnit + tid, kPointThreads);
+      },
+      [&](const BinSegment& S, int n, int units) {
+        __threadfence();  // this block's counts and words before its units are counted
+        __syncthreads();
+        if (tid == 0) s_done = atomicAdd(&S.bin_off[KF_NBINS], n) + n;
+        __syncthreads();
+        if (s_done != units) return;
+        __threadfence();
+        int carry = 0;
+        bool over = false;  // a bin with places that do not fit their words
+        for (int b0 = 0; b0 < KF_NBINS; b0 += 4 * kPointThreads) {
+          int v[4], sum = 0;
+#pragma unroll
+          for (int t = 0; t < 4; ++t) {
+            v[t] = __ldcg(&S.bin_off[b0 + 4 * tid + t]);
+            over |= v[t] > int(kPlaceMax);
+            sum += v[t];
+          }
+          int inc = sum;
+#pragma unroll
+          for (int d = 1; d < 32; d *= 2) {
+            const int o = __shfl_up_sync(0xffffffffu, inc, d);
+            if (lane >= d) inc += o;
+          }
+          if (lane == 31) s_sum[warp] = inc;
+          __syncthreads();
+          int at = carry + inc - sum;
+          for (int w = 0; w < kPointThreads / 32; ++w) {
+            if (w < warp) at += s_sum[w];
+            carry += s_sum[w];
+          }
+#pragma unroll
+          for (int t = 0; t < 4; ++t) {
+            S.bin_off[b0 + 4 * tid + t] = at;
+            at += v[t];
+          }
+          __syncthreads();  // s_sum is read before the next bins'
+        }
+        if (tid == 0) S.bin_off[KF_NBINS] = carry;
+        if (__syncthreads_or(over))
+          for (int64_t q = S.p0 + tid; q < S.p1; q += kPointThreads) {
+            const uint32_t w = uint32_t(__ldcg(&S.out_id[q]));
+            if ((w & kPlaceMax) != kPlaceMax) continue;
+            const uint32_t place = __float_as_uint(__ldcg(&S.out_pts[q].x));
+            S.out_id[q] = int(kIsPosition | (uint32_t(S.bin_off[w >> kPlaceBits]) + place));
+          }
+      });
+}
+
+__global__ void __launch_bounds__(kPointThreads)
+    bin_large_place_kernel(const __grid_constant__ BinArgs A, const int64_t limit) {
+  chain_begin();
+  for_large<kPointThreads>(
+      A, limit, [](int64_t points) { return (points + kLargeUnit - 1) / kLargeUnit; },
+      [&](int, const BinSegment& S, int64_t u) {
+        place_points<false, kLargePer>(S, S.p0 + u * kLargeUnit + int(threadIdx.x), kPointThreads);
+      },
+      [](const BinSegment&, int, int) {});
+}
+
+// As bin_order_kernel, with bins of about a run's worth a warp at each segment's
+// own density.
+__device__ __forceinline__ int large_bins(int64_t points) {
+  return points * 32 <= 2 * int64_t(kOrderRun) * KF_NBINS ? 32 : 8;
+}
+__global__ void __launch_bounds__(32 * kOrderWarps, 8)
+    bin_large_order_kernel(const __grid_constant__ BinArgs A, const int64_t limit) {
+  chain_begin();
+  __shared__ int s_id[kOrderWarps][kOrderRun];
+  __shared__ int s_off[kOrderWarps][33];
+  const int warp = threadIdx.x >> 5;
+  for_large<32 * kOrderWarps>(
+      A, limit, [](int64_t points) { return KF_NBINS / (large_bins(points) * kOrderWarps); },
+      [&](int s, const BinSegment& S, int64_t u) {
+        const int at = int(u) * kOrderWarps + warp;
+        if (large_bins(S.p1 - S.p0) == 32)
+          order_bins<32, false>(A, s, kNoLimit, at * 32, s_id[warp], s_off[warp]);
+        else
+          order_bins<8, false>(A, s, kNoLimit, at * 8, s_id[warp], s_off[warp]);
+        __syncwarp();  // off is read before the next unit's
+      },
+      [](const BinSegment&, int, int) {});
+}
+
 constexpr int kMaxDevices = 64;
 
 // a kernel's shared-memory attributes, set once per device (the serving loop
@@ -510,6 +718,19 @@ static cudaError_t launch_bin_wide(const BinArgs& a, cudaStream_t st) {
   return e;
 }
 
+// a block per segment; those of more than `limit` points (FINE: no limit) by passes of their own
+template <bool FINE>
+static cudaError_t launch_bin_blocks(const BinArgs& a, int64_t limit, int num_sms, cudaStream_t st) {
+  static std::atomic<bool> attr_set[kMaxDevices];
+  constexpr int smem = FINE ? kFineSmem : kScanSmem;
+  cudaError_t e = segment_smem_attrs(bin_segment_kernel<FINE>, smem, attr_set);
+  if (e == cudaSuccess) e = launch_chained(bin_segment_kernel<FINE>, a.n_seg, kScanThreads, smem, st, a, limit);
+  if (e != cudaSuccess || limit == kNoLimit) return e;
+  e = launch_chained(bin_large_count_kernel, 4 * num_sms, kPointThreads, 0, st, a, limit);
+  if (e == cudaSuccess) e = launch_chained(bin_large_place_kernel, 4 * num_sms, kPointThreads, 0, st, a, limit);
+  return e;
+}
+
 cudaError_t launch_bin_segment_table(const BinSegment* table, int n, int64_t n_points, bool fine, cudaStream_t st) {
   if (n <= 0) return cudaSuccess;
   BinArgs a;
@@ -527,50 +748,62 @@ cudaError_t launch_bin_segment_table(const BinSegment* table, int n, int64_t n_p
 // a warp: 350 segments of 20 000 hits 207, 202, 227 and 418 us, 1 540 of 1 000
 // 124, -, 283 and 861; 7 of 20 000 26.8, -, 21.6 and 23.7; one of 1 500 000
 // 1 456, -, 405 and 140.
-static cudaError_t launch_bin_order(const BinArgs& a, int num_sms, bool wide, cudaStream_t st) {
-  const auto go = [&](void (*kernel)(BinArgs), int nb) {
-    return launch_chained(kernel, unsigned(a.n_seg) * unsigned(KF_NBINS / nb / kOrderWarps), 32 * kOrderWarps, 0, st,
-                          a);
+static cudaError_t launch_bin_order(const BinArgs& a, int num_sms, bool wide, int64_t limit, cudaStream_t st) {
+  const auto go = [&](void (*kernel)(BinArgs, int64_t), int nb) {
+    return launch_chained(kernel, unsigned(a.n_seg) * unsigned(KF_NBINS / nb / kOrderWarps), 32 * kOrderWarps, 0, st, a,
+                          limit);
   };
   const auto fills = [&](int nb) { return int64_t(a.n_seg) * (KF_NBINS / nb) >= int64_t(num_sms) * 20; };
   const auto one_run = [&](int nb) { return a.n_points * nb <= int64_t(a.n_seg) * kOrderRun * KF_NBINS; };
-  if (!wide && fills(128) && one_run(128)) return go(bin_order_kernel<128>, 128);
-  if (!wide && fills(64) && one_run(64)) return go(bin_order_kernel<64>, 64);
-  if (fills(32)) return go(bin_order_kernel<32>, 32);
-  return go(bin_order_kernel<8>, 8);
+  if (limit != kNoLimit) {  // blocks for a run each, if all hits were in large segments
+    const int grid = int(std::min<int64_t>(8 * num_sms, a.n_points / (kOrderRun * kOrderWarps) + 1));
+    const cudaError_t e = launch_chained(bin_large_order_kernel, grid, 32 * kOrderWarps, 0, st, a, limit);
+    if (e != cudaSuccess) return e;
+  }
+  const bool all = limit == kNoLimit;
+  if (!wide && fills(128) && one_run(128))
+    return all ? go(bin_order_kernel<128, false>, 128) : go(bin_order_kernel<128, true>, 128);
+  if (!wide && fills(64) && one_run(64))
+    return all ? go(bin_order_kernel<64, false>, 64) : go(bin_order_kernel<64, true>, 64);
+  if (fills(32)) return all ? go(bin_order_kernel<32, false>, 32) : go(bin_order_kernel<32, true>, 32);
+  return go(bin_order_kernel<8, false>, 8);  // (never with a limit: a few segments of over 3 000 hits)
 }
 
-// Which form: one block per segment costs about 10 us plus 1.3 us per 1 000
-// hits of the largest segment, times the rounds of segments on the SMs; the
-// wide passes 20 us plus 0.024 us per 1 000 hits of all segments (measured:
-// 350 segments of 20 000 hits 158 against 185 us, by sub-bin 182 against 210;
-// 28 of 3 000: 18 against 24; 7 of 20 000: 35 against 24; 7 of 200 000: 285
-// against 48; 84 uneven ones of 23 000 on average: 132 against 66).  The sizes
-// are on the device, so the rule goes by their mean: blocks for many segments,
-// among which a large one weighs little, and for small ones.
-static bool one_block_a_segment(const BinArgs& a, int num_sms) {
-  return !a.out_pts || a.n_points <= int64_t(a.n_seg) * (a.n_seg >= num_sms ? 40000 : 3000);
+// Which form: with m thousand hits in the largest segment and n in all, a block
+// per segment takes some 10 + 1.42 m us (by sub-bin 12.5 + 1.5 m), the wide
+// passes 15 + 0.05 a segment + 0.0225 n (20 + 0.07 a segment + 0.0225 n).  7
+// segments of 20 000: 40 against 18 us, of 3 000 15 against 16; 70 of 12 000 27
+// against 36; 350 of 20 000 164 against 190, by sub-bin 186 against 220; 84 uneven
+// ones of 43 000 on average (2 000 ... 200 000) 304 against 102.  The sizes are on
+// the device, so the rule goes by their mean, as if some segment had several
+// times that: blocks for small segments and, up to some 40 000 hits, for more
+// segments than SMs.
+//
+// In the ordered form the segments larger than `limit`, whose block alone would
+// take twice as long as all by the wide passes, are taken from the blocks to
+// passes of their own.  154 segments, half of 1 500 000 hits in 7 of them: 105 us
+// (by blocks alone 195); one of 700 000 hits among 153 of 2 000: 104 (1 240).  A
+// request of up to 150 000 hits, which those passes would cost up to a third,
+// goes without: at most some 0.25 ms, were all in one segment.
+struct BinPlan {
+  bool wide;
+  int64_t limit;
+};
+static BinPlan plan_of(const BinArgs& a, int num_sms) {
+  if (!a.out_pts) return {false, kNoLimit};
+  if (a.n_points > int64_t(a.n_seg) * (a.n_seg >= num_sms ? 40000 : 3000)) return {true, kNoLimit};
+  const int64_t limit = int64_t((10000 + 100.0 * a.n_seg + 0.045 * double(a.n_points)) / 1.42);
+  return {false, !a.unordered && a.n_points > std::max<int64_t>(limit, 150000) ? limit : kNoLimit};
 }
 
 cudaError_t launch_bin_points(const BinArgs& a, int num_sms, cudaStream_t st) {
   if (a.n_seg <= 0) return cudaSuccess;
   if (a.fine_off && !a.unordered) return cudaErrorInvalidValue;  // sub-bins only with the unordered binning
-  cudaError_t e;
-  const bool wide = !one_block_a_segment(a, num_sms);
-  if (wide) {
-    e = a.fine_off ? launch_bin_wide<true>(a, st) : launch_bin_wide<false>(a, st);
-  } else {
-    static std::atomic<bool> seg_attr_set[kMaxDevices], fine_attr_set[kMaxDevices];
-    if (a.fine_off) {
-      e = segment_smem_attrs(bin_segment_kernel<true>, kFineSmem, fine_attr_set);
-      if (e == cudaSuccess) e = launch_chained(bin_segment_kernel<true>, a.n_seg, kScanThreads, kFineSmem, st, a);
-    } else {
-      e = segment_smem_attrs(bin_segment_kernel<false>, kScanSmem, seg_attr_set);
-      if (e == cudaSuccess) e = launch_chained(bin_segment_kernel<false>, a.n_seg, kScanThreads, kScanSmem, st, a);
-    }
-  }
-  if (e == cudaSuccess && !a.unordered && a.n_points > 0)
-    e = launch_bin_order(a, num_sms, wide, st);
+  const BinPlan plan = plan_of(a, num_sms);
+  cudaError_t e = plan.wide ? (a.fine_off ? launch_bin_wide<true>(a, st) : launch_bin_wide<false>(a, st))
+                            : (a.fine_off ? launch_bin_blocks<true>(a, plan.limit, num_sms, st)
+                                          : launch_bin_blocks<false>(a, plan.limit, num_sms, st));
+  if (e == cudaSuccess && !a.unordered && a.n_points > 0) e = launch_bin_order(a, num_sms, plan.wide, plan.limit, st);
   return e;
 }
 
