@@ -731,12 +731,22 @@ static cudaError_t launch_bin_blocks(const BinArgs& a, int64_t limit, int num_sm
   return e;
 }
 
-cudaError_t launch_bin_segment_table(const BinSegment* table, int n, int64_t n_points, bool fine, cudaStream_t st) {
+// The form by the costs given at plan_of, the sizes being known here (a request
+// served alone mostly has small segments: with the wide passes whatever the size a
+// small event's latency was 201 us, not 193).
+cudaError_t launch_bin_segment_table(const BinSegment* table, int n, int64_t n_points, int64_t max_points, bool fine,
+                                     int num_sms, cudaStream_t st) {
   if (n <= 0) return cudaSuccess;
   BinArgs a;
   a.table = table;
   a.n_seg = n;
   a.n_points = n_points;
+  const double m = 1e-3 * double(max_points), rounds = double((n + num_sms - 1) / num_sms);
+  const double blocks = rounds * (fine ? 12.5 + 1.5 * m : 10 + 1.42 * m);
+  const double wide = (fine ? 20 + 0.07 * n : 15 + 0.05 * n) + 0.0225e-3 * double(n_points);
+  if (blocks <= wide)
+    return fine ? launch_bin_blocks<true>(a, kNoLimit, num_sms, st)
+                : launch_bin_blocks<false>(a, kNoLimit, num_sms, st);
   return fine ? launch_bin_wide<true>(a, st) : launch_bin_wide<false>(a, st);
 }
 

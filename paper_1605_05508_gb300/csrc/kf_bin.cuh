@@ -68,9 +68,10 @@ struct BinArgs {
                                       // when set the points are ordered by sub-bin
 };
 
-// Bin the n segments of a device table, n_points points in all (unordered;
-// fine: by sub-bin, every entry's fine_off set).
-cudaError_t launch_bin_segment_table(const BinSegment* table, int n, int64_t n_points, bool fine, cudaStream_t st);
+// Bin the n segments of a device table, n_points points in all, at most
+// max_points in one (unordered; fine: by sub-bin, every entry's fine_off set).
+cudaError_t launch_bin_segment_table(const BinSegment* table, int n, int64_t n_points, int64_t max_points, bool fine,
+                                     int num_sms, cudaStream_t st);
 
 // Sort the points of every segment of `a` into bins (one or several launches on
 // `st`).  out_pts null (seeds): the ids only, unordered, one block per segment.

@@ -387,7 +387,7 @@ static cudaError_t prepare_batch(Serve* sv, const std::vector<Request*>& rs) {
   char* dslot = sv->d_table + kTableBytes * kRing + kPrepBytes * size_t(slot);
   FitEvent* hf = reinterpret_cast<FitEvent*>(hslot);
   BinSegment* hb = reinterpret_cast<BinSegment*>(hslot + kPrepFitBytes);
-  int64_t tracks = 0, points = 0;
+  int64_t tracks = 0, points = 0, most = 0;
   int segs = 0;
   for (size_t k = 0; k < rs.size(); ++k) {
     Request* r = rs[k];
@@ -430,6 +430,7 @@ static cudaError_t prepare_batch(Serve* sv, const std::vector<Request*>& rs) {
       b.p1 = std::min<int64_t>(hoff[l + 1], L.nh);
       b.begin = points;
       points += b.p1 - b.p0;
+      most = std::max(most, b.p1 - b.p0);
       b.bin_off = reinterpret_cast<int32_t*>(d + L.d_boff) + int64_t(l) * (KF_NBINS + 1);
       b.fine_off = L.fine ? reinterpret_cast<int32_t*>(d + L.d_fine) + int64_t(l) * (KF_NBINS_FINE + 1) : nullptr;
       b.out_pts = reinterpret_cast<float4*>(d + L.d_bhits);
@@ -455,7 +456,7 @@ static cudaError_t prepare_batch(Serve* sv, const std::vector<Request*>& rs) {
   fa.mass = ctx->mass;
   e = launch_fit_fused_table(fa, df, int(rs.size()), tracks, s);
   // the build's results do not depend on the order of the hits inside a bin
-  if (e == cudaSuccess) e = launch_bin_segment_table(db, segs, points, sub_bins, s);
+  if (e == cudaSuccess) e = launch_bin_segment_table(db, segs, points, most, sub_bins, ctx->num_sms, s);
   if (e != cudaSuccess) return e;
   // (a register-resident build takes the seeds in their order, from the fit)
   for (size_t k = 0; k < rs.size() && sv->tune.build_scan != 4; ++k) {
