@@ -258,7 +258,7 @@ typedef struct {
  * asc, hit id asc) and only the best max_cands are copied and updated.
  * max_cands = 1 is the best-hit approach.  The window is the set of bins
  * that a hit with chi2 < cut can fall in (chi2 >= (u.r)^2 / (u^T S u) for
- * every direction u), each bound widened by 0.1 % plus 1e-6 rad / 1e-5 cm
+ * every direction u), each bound widened by 0.1 % plus 1.1e-5 rad / 1e-5 cm
  * against rounding, so binning never changes the result.  The
  * register-resident layout (kf_tuning.build_scan 4) takes the seeds in their
  * given order, the others in (eta, phi) bin order within each event; the

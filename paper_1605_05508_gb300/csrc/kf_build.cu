@@ -8,7 +8,7 @@
 //   2. derives the hit window: chi2 >= (u.r)^2 / (u^T S u) for every unit u,
 //      so a hit with chi2 < cut lies within sqrt(cut u^T S u) of the
 //      prediction along the tangent, the normal and z; those bounds, each
-//      widened by 0.1 % plus 1e-6 rad / 1e-5 cm against rounding, are mapped
+//      widened by 0.1 % plus 1.1e-5 rad / 1e-5 cm against rounding, are mapped
 //      to eta x phi bins,
 //   3. computes the chi2 increment of every hit in the window and keeps its
 //      best children in a sorted register list (the bookkeeping list of the
@@ -81,10 +81,10 @@ __device__ __forceinline__ int wrap_phi(int d) {  // to [-KF_BIN_PHI/2, KF_BIN_P
   return ((d + KF_BIN_PHI / 2) & (KF_BIN_PHI - 1)) - KF_BIN_PHI / 2;
 }
 
-// Approximate square root, reciprocal square root (a few ulp) and atan2 (within
-// 3e-6 rad) for the window bounds, which are widened by far more than that:
-// the correctly rounded forms and the library atan2f took several times the
-// instructions and a chain of dependent branches.
+// Approximate square root and reciprocal square root (a few ulp) and atan2
+// (kf::atan2_approx, within 3e-6 rad) for the window bounds, which are widened by
+// far more than that: the correctly rounded forms and the library atan2f took
+// several times the instructions and a chain of dependent branches.
 __device__ __forceinline__ float sqrt_approx(float x) {
   float r;
   asm("sqrt.approx.ftz.f32 %0, %1;" : "=f"(r) : "f"(x));
@@ -95,25 +95,6 @@ __device__ __forceinline__ float rsqrt_approx(float x) {
   asm("rsqrt.approx.ftz.f32 %0, %1;" : "=f"(r) : "f"(x));
   return r;
 }
-// atan on [0, 1] by an odd polynomial of degree 11 (coefficients fitted for
-// the least maximal error, 1.7e-6), extended by the symmetries of atan2.
-// NaN for (0, 0) and non-finite arguments.
-__device__ __forceinline__ float atan2_approx(float y, float x) {
-  const float ax = fabsf(x), ay = fabsf(y);
-  const float t = __fdividef(fminf(ax, ay), fmaxf(ax, ay));
-  const float u = t * t;
-  float r = -0.011719135f;
-  r = fmaf(r, u, 0.05264735f);
-  r = fmaf(r, u, -0.11642648f);
-  r = fmaf(r, u, 0.19354038f);
-  r = fmaf(r, u, -0.33262283f);
-  r = fmaf(r, u, 0.9999772f);
-  r = r * t;
-  r = ay > ax ? 0.5f * kPi - r : r;
-  r = x < 0.f ? kPi - r : r;
-  return copysignf(r, y);
-}
-
 // Window of a predicted candidate: the eta rows
 // e0..e1 and phi bins fa0..fa1, fb0..fb1 (second part when the window wraps
 // around phi = +-pi) that can hold a hit with chi2 < cut at radius R; the
@@ -144,7 +125,7 @@ __device__ __forceinline__ void hit_window(const float p[6], const float lo[3], 
   // (x >= 0), a bound from above.
   constexpr float kWiden = 1.001f;
   const float rin = R - wn * kWiden;
-  const float phic = atan2_approx(Y, X);
+  const float phic = kf::atan2_approx(Y, X);
   const float dphi =
       (rin > 0.5f * R && wt * kWiden < rin) ? __fdividef(wt * kWiden, rin) * kWiden + 1.1e-5f : 10.f;
   if (dphi < 1.f && phic >= -kPi && phic <= kPi) {  // also false for NaN

@@ -86,6 +86,26 @@ KF_HD float div_fast(float a, float b) {
 }
 KF_HD double div_fast(double a, double b) { return a / b; }
 
+// atan2 within 3e-6 rad: atan on [0, 1] by the odd minimax polynomial of degree
+// 11 (Remez exchange; its error reaches 1.68e-6 with alternating signs at seven
+// points), extended by the symmetries of atan2.  NaN for (0, 0); of an infinite
+// or NaN argument it may make any angle.
+KF_HD float atan2_approx(float y, float x) {
+  const float ax = fabsf(x), ay = fabsf(y);
+  const float t = div_fast(fminf(ax, ay), fmaxf(ax, ay));
+  const float u = t * t;
+  float r = -0.011719135f;
+  r = fmaf(r, u, 0.05264735f);
+  r = fmaf(r, u, -0.11642648f);
+  r = fmaf(r, u, 0.19354038f);
+  r = fmaf(r, u, -0.33262283f);
+  r = fmaf(r, u, 0.9999772f);
+  r = r * t;
+  r = ay > ax ? 1.57079632679489661923f - r : r;
+  r = x < 0.f ? 3.14159265358979323846f - r : r;
+  return copysignf(r, y);
+}
+
 // ---- pairs: two single-precision operations in one instruction on sm_103a,
 // each rounded as by itself (so the bits are those of two scalar ones).  A
 // three-register fused multiply-add is bound by the reads of its operands (46
