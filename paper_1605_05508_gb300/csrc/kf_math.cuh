@@ -251,8 +251,9 @@ KF_HD constexpr bool jnz(int i, int l) { return i < 5 && l != 2; }
 // Newton steps and the final point (the same evaluations, so the same bits):
 // smaller code, for kernels that wait on instruction fetch (the build: 1 182
 // against 1 202 us a 50 x 5 000-seed step; the fit, which does not, takes
-// 1 459 against 1 443 us for 4M tracks with it).
-template <typename T, int NEWTON, bool EXT, bool LEAN = false>
+// 1 459 against 1 443 us for 4M tracks with it).  PAIRS: the Jacobian and its
+// product with C on pairs of rows (single precision; without, for tests).
+template <typename T, int NEWTON, bool EXT, bool LEAN = false, bool PAIRS = !Lanes<T>::kDouble>
 KF_HD typename Lanes<T>::I propagate_lanes(T p[6], T lo[3], T C[21], T a, T R, typename Lanes<T>::M live) {
   using M = typename Lanes<T>::M;
   using I = typename Lanes<T>::I;
@@ -376,7 +377,7 @@ KF_HD typename Lanes<T>::I propagate_lanes(T p[6], T lo[3], T C[21], T a, T R, t
   // C' = J C J^T with T1 = J C (rows 0..4; row 5 of J is e_pz, and J[i][2] =
   // (i == 2))
   T J[5][6], T1[5][6];
-  if constexpr (!Lanes<T>::kDouble) {
+  if constexpr (PAIRS) {
     // ---- surface Jacobian and T1 = J C as below, rows (0, 1) and (3, 4) in
     // pairs, every element by the same operations in the same order
     const float ip2 = ip * ip;
