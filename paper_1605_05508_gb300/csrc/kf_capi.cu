@@ -200,6 +200,7 @@ static int fit_staged(kf_ctx* ctx, const kf_tracks* seeds, const kf_track_hits* 
   const int64_t n = seeds->n;
   const int L = hits->n_layers;
   *done = false;
+  if (!stage_layout_ok(seeds, hits, out)) return KF_OK;  // before any scratch: the fused launch needs none
   int32_t* st = status;
   if (!st) {
     const int rc = scratch_reserve(ctx, ctx->s_status, size_t(n) * sizeof(int32_t));

@@ -140,7 +140,7 @@ __device__ __forceinline__ void fit_layer_track(const FitLayerArgs& A, int64_t i
 // registers.  Completion is tracked by one mbarrier per buffer; every wait is
 // bounded (a wait that gives up marks the warp's remaining tracks with
 // KF_ST_DEVICE_TIMEOUT).  Requires n, begin and count multiples of 32 and
-// 16-byte aligned rows; kf_fit falls back to fit_layer_kernel otherwise.
+// 16-byte aligned rows (stage_layout_ok); kf_fit takes the fused launch otherwise.
 constexpr int kStageTile = 32;                 // tracks per warp tile
 constexpr int kStageThreads = 64;              // two warps per block
 constexpr int kStageBlocksPerSM = 12;          // 24 warps per SM
@@ -443,6 +443,19 @@ __global__ void __launch_bounds__(kFitThreads) fit_f64_kernel(const FitF64Args A
   if (A.first || raised || A.last) A.status[i] = st;
 }
 
+static bool stage_aligned(const void* p) { return (reinterpret_cast<uintptr_t>(p) & 15u) == 0; }
+
+bool stage_layout_ok(const kf_tracks* seeds, const kf_track_hits* hits, const kf_tracks* out) {
+  if (seeds->n % kStageTile || seeds->n > (int64_t(1) << 31) - 1) return false;
+  const float* const in[] = {seeds->par, seeds->par_lo, seeds->cov, hits->xyz};
+  for (const float* p : in)
+    if (!stage_aligned(p)) return false;
+  if (hits->n_layers > 1)  // the layers after the first read the outputs
+    for (const float* p : {out->par, out->par_lo, out->cov})
+      if (!stage_aligned(p)) return false;
+  return true;
+}
+
 // Tensor maps of a layer step for fit_layer_stage_kernel: 2-D views (x =
 // track, y = row) of the input state, position low parts, covariance and the
 // layer's hits, boxes of 32 tracks x all rows.  False when the layout does not
@@ -451,8 +464,8 @@ __global__ void __launch_bounds__(kFitThreads) fit_f64_kernel(const FitF64Args A
 bool make_stage_maps(const FitLayerArgs& a, FitStageMaps* m) {
   if (a.n % kStageTile || a.begin % kStageTile || a.count % kStageTile || a.count <= 0) return false;
   if (a.n > (int64_t(1) << 31) - 1) return false;
-  auto aligned = [](const void* p) { return (reinterpret_cast<uintptr_t>(p) & 15u) == 0; };
-  if (!aligned(a.in_par) || !aligned(a.in_cov) || !aligned(a.hit) || (a.in_lo && !aligned(a.in_lo))) return false;
+  for (const float* p : {a.in_par, a.in_cov, a.hit, a.in_lo})
+    if (!stage_aligned(p)) return false;
   static PFN_cuTensorMapEncodeTiled_v12000 encode = nullptr;
   static std::once_flag once;
   std::call_once(once, [] {

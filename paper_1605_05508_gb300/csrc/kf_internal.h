@@ -200,8 +200,10 @@ FitFusedArgs fused_args(const kf_ctx* ctx, const kf_tracks* seeds, const kf_trac
 // block: threads per block, 64 or 128 (kf_tuning.fit_block)
 cudaError_t launch_fit_fused(const FitFusedArgs& a, int block, cudaStream_t st);
 cudaError_t launch_fit_mixed(const FitFusedArgs& a, cudaStream_t st);
-// staged layer step (kf_tuning.fit_stage): false from make_stage_maps when the
-// batch's layout does not allow it (kf_fit then takes the fused launch)
+// staged layer step (kf_tuning.fit_stage): false from stage_layout_ok (a batch),
+// or make_stage_maps (one step of it), when the layout does not allow it (kf_fit
+// then takes the fused launch)
+bool stage_layout_ok(const kf_tracks* seeds, const kf_track_hits* hits, const kf_tracks* out);
 bool make_stage_maps(const FitLayerArgs& a, FitStageMaps* m);
 cudaError_t launch_fit_layer_stage(const FitLayerArgs& a, const FitStageMaps& m, int num_sms, cudaStream_t st);
 // One event of a table-driven fused fit: its arrays, as in FitFusedArgs, and
