@@ -1,4 +1,6 @@
-"""The forms of the fit: what each asks of the context's device memory."""
+"""The fit in one launch and the staged launches per layer give the same bits
+(batches whose layout the staged form takes, so that the two differ in every
+launch), and what each asks of the context's device memory."""
 import pytest
 
 from paper_1605_05508_gb300 import synth as S
@@ -28,6 +30,20 @@ def _run(ctx, fn, ev, valid, lo=True, status=True):
     fn(ctx, s, h, o, chi2, st)
     torch.cuda.synchronize()
     return [t for t in (o.par, o.par_lo, o.cov, chi2, st) if t is not None], free - torch.cuda.mem_get_info()[0]
+
+
+@pytest.mark.parametrize("n,chunk", [(32, 0), (4096, 0), (40_000, 0), (300_032, 262144)])
+def test_one_launch_equals_staged_launches(cuda_ctx_factory, n, chunk):
+    import torch
+    from paper_1605_05508_gb300 import kf
+    ctx = cuda_ctx_factory(S.barrel().radii)
+    ev, valid = _batch(n)
+    kf.kf_set_tuning(ctx, 64, 0, 8, 4, chunk, 1)
+    staged, _ = _run(ctx, kf.kf_fit, ev, valid)
+    kf.kf_set_tuning(ctx, 128, 0, 8, 4, 0, 0)
+    for fn in (kf.kf_fit, kf.kf_fit_fused, kf.kf_fit_noalloc)[:3 if n <= kf.NOALLOC_MAX_TRACKS else 2]:
+        for a, b in zip(_run(ctx, fn, ev, valid)[0], staged):
+            assert torch.equal(a, b)
 
 
 def test_the_single_launch_takes_no_device_memory(cuda_ctx_factory):
