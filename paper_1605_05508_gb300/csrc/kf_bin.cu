@@ -187,7 +187,6 @@ __device__ __forceinline__ void bin_one_segment(const BinSegment& S, int32_t* ou
         if (out_pts) {  // the bin from the first pass; out_id stays scratch
           const int64_t q = p0 + atomicAdd(&cnt[pad_idx(bins[u])], 1);
           out_pts[q] = make_float4(x[u], y[u], z[u], __int_as_float(i));
-          if (out_seg) out_seg[q] = seg;
         } else {
           const int64_t q = p0 + atomicAdd(&cnt[pad_idx(bin_of<NPHI>(x[u], y[u], z[u]))], 1);
           out_id[q] = i;
@@ -809,6 +808,7 @@ static BinPlan plan_of(const BinArgs& a, int num_sms) {
 cudaError_t launch_bin_points(const BinArgs& a, int num_sms, cudaStream_t st) {
   if (a.n_seg <= 0) return cudaSuccess;
   if (a.fine_off && !a.unordered) return cudaErrorInvalidValue;  // sub-bins only with the unordered binning
+  if (a.out_seg && a.out_pts) return cudaErrorInvalidValue;      // segments only with ids
   const BinPlan plan = plan_of(a, num_sms);
   cudaError_t e = plan.wide ? (a.fine_off ? launch_bin_wide<true>(a, st) : launch_bin_wide<false>(a, st))
                             : (a.fine_off ? launch_bin_blocks<true>(a, plan.limit, num_sms, st)

@@ -62,7 +62,7 @@ struct BinArgs {
   float4* out_pts = nullptr;          // [total] or null
   int32_t* out_id = nullptr;          // [total] required: id within the segment, bin order (with
                                       // out_pts: scratch, each point's bin and place in input order)
-  int32_t* out_seg = nullptr;         // [total] or null
+  int32_t* out_seg = nullptr;         // without out_pts: [total] the segment of each id, or null
   int unordered = 0;                  // 1: leave each bin in scatter order (no sort by id)
   int32_t* fine_off = nullptr;        // unordered only: [n_seg][KF_NBINS_FINE + 1] sub-bin starts, or null;
                                       // when set the points are ordered by sub-bin
