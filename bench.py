@@ -240,9 +240,13 @@ def ncu_traffic(n_tracks):
     return None if b is None else b * n_tracks
 
 
-# FP32 work of one track-layer step (FFMA x 2 + FADD + FMUL thread
-# instructions of the fused fit, counted by ncu).
+# FP32 work of one track-layer step: the operations of the scalar form of the
+# fit (FFMA x 2 + FADD + FMUL thread instructions counted by ncu when the kernel
+# had that form).  The kernel does the same operations, part of them two an
+# instruction, which those counters do not see, so the count is carried over.
 FIT_FLOP_PER_TRACK_LAYER = 1441.9
+FIT_FLOP_SOURCE = ("operations of the scalar form of the same arithmetic (FFMA x 2 + FADD + FMUL thread instructions "
+                   "counted by ncu on it); the kernel's two-wide instructions are not in those counters")
 
 # Algorithmic bytes of one track-layer step of the per-layer fit as the method
 # needs them: read the state (par 24 + cov 84), the hit (12) and the charge (1),
@@ -354,7 +358,7 @@ def run_ours(a):
         roof = staged_roofline(n, L, chunks, ms_per_step)
     else:  # one launch, the state in registers: bound by the FP32 pipe
         roof = dict(fp32_roofline(FIT_FLOP_PER_TRACK_LAYER, n * L, ms_per_step / 1e3, line_peaks,
-                                  "FFMA x 2 + FADD + FMUL thread instructions counted by ncu"),
+                                  FIT_FLOP_SOURCE),
                     kernel=f"fit_fused_kernel<{tuning['fit_block']}>", launch_us=ms_per_step * 1e3)
 
     line = {"metric": METRIC, "value": value, "unit": UNIT, "n_gpus": world, "steps": a.steps,
@@ -440,15 +444,15 @@ def chi2_error_table(g_chi2, o_chi2):
 
 
 def fp32_roofline(flop_per_unit, units, seconds, peaks, source):
-    """FP32 flop fraction of the measured FP32 peak for a kernel whose FP32
-    instruction counts per unit come from a committed ncu summary."""
+    """FP32 flop fraction of the measured FP32 peak for a kernel, its operation
+    count per unit from `source`."""
     if not flop_per_unit or not peaks or not peaks.get("fp32_tflops"):
         return None
     ach = flop_per_unit * units / seconds
     return {"bound": "fp32", "achieved": ach / 1e12, "peak": peaks["fp32_tflops"], "unit": "TFLOP/s",
             "frac": ach / (peaks["fp32_tflops"] * 1e12), "flop_per_unit": flop_per_unit,
             "peak_kind": "measured (kf_measure_peak)",
-            "flop_source": f"ncu FFMA x2 + FADD + FMUL thread instructions ({source})"}
+            "flop_source": source}
 
 
 def extras(a, ctx, kf, torch, dev, det, ev, seeds, hits, out, chi2, status, stream, value, ms_per_step, rank, world,
@@ -484,8 +488,7 @@ def extras(a, ctx, kf, torch, dev, det, ev, seeds, hits, out, chi2, status, stre
                                     "unit": "warp instructions/s", "frac": ach / peak,
                                     "warp_instructions_per_track_layer": ipt,
                                     "peak_kind": "4 issues per SM per cycle x SMs x max SM clock"}
-    fpt = profile_value("fit_fused_kernel.instructions.txt", "fp32_flop_per_track_layer")
-    f32r = fp32_roofline(fpt, n * L, ms_f / 1e3, peaks, "profiles/fit_fused_kernel.instructions.txt")
+    f32r = fp32_roofline(FIT_FLOP_PER_TRACK_LAYER, n * L, ms_f / 1e3, peaks, FIT_FLOP_SOURCE)
     if f32r:
         res["fused"]["fp32_roofline"] = dict(f32r, kernel="fit_fused_kernel")
 
@@ -630,14 +633,24 @@ def build_kernel_name(t, max_cands):
     return f"build_step_kernel<{t['build_hit_tile']}, {lw}, {int(scan == 1)}>"
 
 
-def build_step_launches(tune, Lb, max_cands):
-    """Kernel launches of one build step of many segments: the seed fit (one),
-    the hit binning (one block a segment; ordered, the order by id too) and
-    kf_build -- register-resident: with more than one lane a seed the first
+def binning_launches(unordered, n_seg, n_hits, num_sms):
+    """Kernel launches of kf_bin_hits, by the library's rule (plan_of in
+    kf_bin.cu): passes over all hits (zero, count, scan, place) or a block a
+    segment, ordered with the passes for large segments and the order by id."""
+    order = 0 if unordered or n_hits == 0 else 1
+    if n_hits > n_seg * (40000 if n_seg >= num_sms else 3000):
+        return 4 + order
+    large = order and n_hits > max((10000 + 100 * n_seg + 0.045 * n_hits) / 1.42, 150000)
+    return 1 + order + (3 if large else 0)
+
+
+def build_step_launches(tune, Lb, max_cands, n_seg, n_hits, num_sms):
+    """Kernel launches of one build step: the seed fit (one), the hit binning
+    and kf_build -- register-resident: with more than one lane a seed the first
     layer, the other layers and the covariance check, else the seeds' events
     and the layers; else the seed ordering, global ids, first candidates, the
     layer steps and the final selection."""
-    binning = 1 if tune.get("bin_unordered") else 2
+    binning = binning_launches(tune.get("bin_unordered"), n_seg, n_hits, num_sms)
     if tune["build_scan"] == 4:
         build = 3 if max_cands > 1 else 2
     else:
@@ -894,7 +907,8 @@ def build_leg(a, kf, torch, dev, stream, rank, world, dist, peaks=None):
            "bin_order": "scatter order inside each bin (bin_unordered 1; the build's results are the same bits)"
                         + ("; by 64 x 512 sub-bins, whose starts the register-resident build's windows look up"
                            if fine is not None else ""),
-           "gpu_launches_per_step": build_step_launches(tune6, Lb, 6)}
+           "gpu_launches_per_step": build_step_launches(tune6, Lb, 6, E * Lb, int(batch.layer_xyz.shape[1]),
+                                                        torch.cuda.get_device_properties(dev).multi_processor_count)}
     # roofline of the build by the method's bytes: per seed and layer ~6 parents
     # read (112 B of state each), ~6 children written (112 B + a 4 B hit id) and
     # the hits of their windows, ~1.4 kB; over the build phase's CUDA-event time
@@ -933,7 +947,7 @@ def build_leg(a, kf, torch, dev, stream, rank, world, dist, peaks=None):
                                             prof, "active_lanes_per_warp_instruction", BUILD_SOURCES),
                                         "peak_kind": "4 issues per SM per cycle x SMs x max SM clock"}
         f32r = fp32_roofline(profile_value(prof, "fp32_flop_per_build", BUILD_SOURCES), 1, t_build, peaks,
-                             f"profiles/{prof}")
+                             f"ncu FFMA x 2 + FADD + FMUL thread instructions (profiles/{prof})")
         if f32r:
             res["roofline"]["counted_fp32"] = f32r
     # DRAM bytes of kf_build's launches (one ncu capture of the same setting,
