@@ -158,7 +158,10 @@ constexpr int kResThreads = 128;
 constexpr int kResBlocksPerSM = 4;
 // resident blocks per SM of build_resident_kernel<W>: 5 (96 registers a
 // thread; at W = 6 with the covariance arithmetic on pairs of rows 1 052
-// against 1 061 us a 50-event step with 4, before that 6 % slower), 4 at W = 8
+// against 1 061 us a 50-event step with 4, before that 6 % slower), 4 at W = 8.
+// The served form, which spills some 100 bytes at 5, serves the same events per
+// second at either (11 440 at saturation from one thread, 11 300 and 11 575 from
+// four, runs differing by 3 %).
 constexpr int resident_blocks_per_sm(int W) { return W <= 6 ? 5 : kResBlocksPerSM; }
 // One batch of seeds of a register-resident build: the whole batch of a
 // kf_build call, or one served event.
@@ -216,7 +219,7 @@ inline int resident_lanes(int max_cands) {
   return max_cands <= 2 ? max_cands : max_cands <= 4 ? 4 : max_cands <= 6 ? 6 : 8;
 }
 // With several lanes a seed, the resident layout leaves the best covariance's
-// positive-definiteness check to the final kernel (paths_only = 2).
+// positive-definiteness check to the final kernel (bit 1 of BuildFinalArgs::rest).
 inline bool resident_defers_pd(int max_cands) { return resident_lanes(max_cands) > 1; }
 // The history of a group's candidates stays in shared memory for up to this
 // many building layers, and build_resident_kernel then writes the best paths

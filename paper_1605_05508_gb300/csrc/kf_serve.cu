@@ -9,8 +9,8 @@
 //     block of the device arena are free (memory-based admission),
 //   * prepares the events admitted in one iteration together, on one of
 //     several preparation streams: their input copies, then one seed-fit
-//     launch over all their seeds and one binning launch over all their hit
-//     segments (and for the layer-stepping layouts each event's seed
+//     launch over all their seeds and the binning of all their hit segments
+//     in the same launches (and for the layer-stepping layouts each event's seed
 //     ordering and first candidates),
 //   * issues ONE build-step launch per iteration over every resident event,
 //     each at its own layer (the slot table tells each block its event,

@@ -282,8 +282,8 @@ def kf_fit_host(ctx, seeds: Tracks, hits: TrackHits, out: Tracks, chi2=None, sta
 
 
 def kf_fit_noalloc(ctx, seeds: Tracks, hits: TrackHits, out: Tracks, chi2=None, status=None, stream=None):
-    """kf_fit with its per-track scratch in libkf's static device memory: no
-    allocation (batches up to NOALLOC_MAX_TRACKS)."""
+    """kf_fit always by the single launch, which needs no scratch: no allocation
+    (batches up to NOALLOC_MAX_TRACKS)."""
     s, h, o = seeds.abi(), hits.abi(), out.abi()
     _check(lib().kf_fit_noalloc(_h(ctx), C.byref(s), C.byref(h), C.byref(o), _ptr(chi2), _ptr(status),
                                 _stream(stream)), "kf_fit_noalloc", _h(ctx))
