@@ -793,7 +793,8 @@ static cudaError_t launch_bin_order(const BinArgs& a, int num_sms, bool wide, in
 // passes of their own.  154 segments, half of 1 500 000 hits in 7 of them: 105 us
 // (by blocks alone 195); one of 700 000 hits among 153 of 2 000: 104 (1 240).  A
 // request of up to 150 000 hits, which those passes would cost up to a third,
-// goes without: at most some 0.25 ms, were all in one segment.
+// goes without: at most some 0.25 ms, were all in one segment.  An unordered one
+// goes without too (its callers have always had a block a segment there).
 struct BinPlan {
   bool wide;
   int64_t limit;
